@@ -43,7 +43,7 @@ __global__ void __launch_bounds__(TX * TY, (512 / (TX * TY)) > 1 ? 512 / (TX * T
             unsigned* __restrict__ next, int k, int trial) {
   using TileT = Tile<TX, TY, S>;
   using T = typename S::T;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
+  extern __shared__ __align__(128) unsigned char smem_raw[];
   auto& sm = *reinterpret_cast<typename TileT::Smem*>(smem_raw);
   __shared__ LatSlot ls;
   __shared__ int s_it;
@@ -69,7 +69,7 @@ __global__ void __launch_bounds__(TX * TY, (512 / (TX * TY)) > 1 ? 512 / (TX * T
     const int kc = w.y / ls.cols, c = w.y - kc * ls.cols;
     const int zb = (int)((long long)kc * ls.L.nz / ls.nch), ze = (int)((long long)(kc + 1) * ls.L.nz / ls.nch);
     t.setup(c % ls.cols_x, c / ls.cols_x);
-    t.run(zb, ze, (kc & 1) != 0);
+    (void)t.run(zb, ze, (kc & 1) != 0);  // per-thread pulls always land
     if (ls.L.geometry != 0) {
       const double e = t.block_evap();
       // a slot per item (batch_build checks that every member has a slot for each
@@ -91,7 +91,7 @@ __global__ void k_batch_advance(LatSlot* __restrict__ lats, int n, int K) {
 template <int TX, int TY, class S>
 cudaError_t launch_batch(const LatSlot* lats, const int2* items, int nitems, unsigned* next, int k, int trial,
                          int grid, cudaStream_t st) {
-  k_batch<TX, TY, S><<<grid, TX * TY, step_smem<TX, TY, S>(), st>>>(lats, items, nitems, next, k, trial);
+  k_batch<TX, TY, S><<<grid, TX * TY, sizeof(typename Tile<TX, TY, S>::Smem), st>>>(lats, items, nitems, next, k, trial);
   return cudaGetLastError();
 }
 
@@ -99,9 +99,9 @@ template <int TX, int TY, class S>
 int occupancy_batch() {
   int nb = 0;
   if (cudaFuncSetAttribute(k_batch<TX, TY, S>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)step_smem<TX, TY, S>()) != cudaSuccess)
+                           (int)sizeof(typename Tile<TX, TY, S>::Smem)) != cudaSuccess)
     return 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_batch<TX, TY, S>, TX * TY, step_smem<TX, TY, S>()) !=
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_batch<TX, TY, S>, TX * TY, sizeof(typename Tile<TX, TY, S>::Smem)) !=
       cudaSuccess)
     return 0;
   return nb;

@@ -14,6 +14,7 @@
 // is index arithmetic.
 #pragma once
 
+#include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
@@ -61,6 +62,31 @@ constexpr float kW0 = 11184812.0f * 0x1p-25f;  // 1 - 12 kW1 exactly
 __host__ __device__ constexpr float wgt(int i) { return i == 0 ? kW0 : (i <= 6 ? kW1 : kW2); }
 __host__ __device__ constexpr double wgt_d(int i) { return i == 0 ? 1.0 / 3.0 : (i <= 6 ? 1.0 / 18.0 : 1.0 / 36.0); }
 
+// ------------------------------------------------------------------ pair arithmetic
+// Both components of a site go through the same operations, so the kernels hold them as
+// pairs V = float2 (r, b) and issue one packed instruction (add / mul / fma .f32x2) for
+// the two: the same correctly rounded result in each half as the scalar operation, half
+// the instructions. V = float runs one component (an odd component of the N-component step).
+__device__ __forceinline__ float vadd(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ float vsub(float a, float b) { return __fsub_rn(a, b); }
+__device__ __forceinline__ float vmul(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ float vfma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+// The builtins keep products and sums apart; add / mul.rn.f32x2 written as inline PTX are
+// contracted by the assembler (measured: 21% of random a b + c differed).
+__device__ __forceinline__ float2 vadd(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 vmul(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 vfma(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+// a - b = (-1) b + a, rounded once
+__device__ __forceinline__ float2 vsub(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.0f, -1.0f), a); }
+__device__ __forceinline__ float vneg(float a) { return -a; }
+__device__ __forceinline__ float2 vneg(float2 a) { return make_float2(-a.x, -a.y); }
+template <class V>
+__device__ __forceinline__ V vset(float a);
+template <>
+__device__ __forceinline__ float vset<float>(float a) { return a; }
+template <>
+__device__ __forceinline__ float2 vset<float2>(float a) { return make_float2(a, a); }
+
 // Everything a launch needs to know about one lattice.
 struct LatDev {
   int nx, ny, nz, nxny;
@@ -96,14 +122,54 @@ __device__ __forceinline__ void cp_async4(uint32_t* smem, const void* gmem) {
   const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
   asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(sa), "l"(gmem) : "memory");
 }
-// 16-byte asynchronous copy kept in L2 only (each row is read once per CTA).
-// Both addresses must be 16-byte aligned.
-__device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
-  const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(sa), "l"(gmem) : "memory");
-}
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
+
+// Bulk copies (the TMA engine) into shared memory, completing on an mbarrier.
+__device__ __forceinline__ unsigned smem_addr(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ void mbar_init(uint64_t* bar, unsigned arrivals) {
+  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(smem_addr(bar)), "r"(arrivals) : "memory");
+  asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+}
+__device__ __forceinline__ void mbar_expect(uint64_t* bar, unsigned bytes) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(smem_addr(bar)), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ bool mbar_try(uint64_t* bar, unsigned parity) {
+  unsigned ok;
+  asm volatile(
+      "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
+      : "=r"(ok)
+      : "r"(smem_addr(bar)), "r"(parity)
+      : "memory");
+  return ok != 0;
+}
+__device__ __forceinline__ unsigned long long global_ns() {
+  unsigned long long t;
+  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+  return t;
+}
+// Waits until the phase of the given parity completes; false when it has not within 2 s.
+__device__ __forceinline__ bool mbar_wait(uint64_t* bar, unsigned parity) {
+  if (mbar_try(bar, parity)) return true;
+  const unsigned long long t0 = global_ns();
+  while (!mbar_try(bar, parity))
+    if (global_ns() - t0 > 2000000000ull) return false;
+  return true;
+}
+// A box of the tensor at element coordinates (x, y, z, i, c); the x start must lie on a
+// 16-byte boundary, parts outside the tensor are filled with zeros.
+__device__ __forceinline__ void tma_load5(void* smem, const CUtensorMap* map, int x, int y, int z, int i, int c,
+                                          uint64_t* bar) {
+  asm volatile(
+      "cp.async.bulk.tensor.5d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5, %6}], "
+      "[%7];\n" ::"r"(smem_addr(smem)),
+      "l"(map), "r"(x), "r"(y), "r"(z), "r"(i), "r"(c), "r"(smem_addr(bar))
+      : "memory");
+}
+// 16-byte asynchronous copy, cached in L2 only; both addresses 16-byte aligned.
+__device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(smem_addr(smem)), "l"(gmem) : "memory");
+}
 
 // ldcg: a population read at L2 only (ld.global.cg), never from L1, for kernels in
 // which other CTAs of the same launch overwrite the data between two reads.
@@ -112,7 +178,7 @@ struct StF32 {
   static __device__ __forceinline__ float ld(const T* p, float) { return __ldg(p); }
   static __device__ __forceinline__ float ldcg(const T* p, float) { return __ldcg(p); }
   static __device__ __forceinline__ float cv(T v, float) { return v; }
-  static __device__ __forceinline__ void st(T* p, float v, float) { *p = v; }
+  static __device__ __forceinline__ void st(T* p, float v, float) { __stcs(p, v); }
   static __device__ __forceinline__ uint32_t pull_async(uint32_t* sm, const T* p) {
     cp_async4(sm, p);
     return 0u;
@@ -169,6 +235,58 @@ struct StBF16 {
   static __device__ __forceinline__ uint32_t pull_async(uint32_t* sm, const T* p) { return pull_async16(sm, p); }
   static __device__ __forceinline__ float word(uint32_t w, uint32_t hi, float wt) {
     return wt + __bfloat162float(__ushort_as_bfloat16((unsigned short)(hi ? w >> 16 : w & 0xffffu)));
+  }
+};
+
+// The pair (r, b) of one direction: decoded from and encoded to the storage type with the
+// single population's operations.
+template <class S>
+struct Pair {
+  using T = typename S::T;
+  static __device__ __forceinline__ float2 cv(T r, T b, float w) { return make_float2(S::cv(r, w), S::cv(b, w)); }
+  static __device__ __forceinline__ void st(T* pr, T* pb, float2 v, float w) {
+    S::st(pr, v.x, w);
+    S::st(pb, v.y, w);
+  }
+};
+template <>
+struct Pair<StF16> {
+  using T = __half;
+  static __device__ __forceinline__ float2 cv(T r, T b, float w) {
+    return vadd(make_float2(w, w), make_float2(__half2float(r), __half2float(b)));
+  }
+  static __device__ __forceinline__ void st(T* pr, T* pb, float2 v, float w) {
+    const float2 h = vsub(v, make_float2(w, w));
+    const __half2 p = __floats2half2_rn(h.x, h.y);
+    *pr = __low2half(p);
+    *pb = __high2half(p);
+  }
+};
+template <>
+struct Pair<StF16S> {
+  using T = __half;
+  static __device__ __forceinline__ float2 cv(T r, T b, float w) {
+    // scalar products: the packed one by a constant was contracted into momentum's differences
+    return make_float2(__fmul_rn(w, __half2float(r)), __fmul_rn(w, __half2float(b)));
+  }
+  static __device__ __forceinline__ void st(T* pr, T* pb, float2 v, float w) {
+    const float2 h = vmul(v, make_float2(1.0f / w, 1.0f / w));
+    const __half2 p = __floats2half2_rn(h.x, h.y);
+    *pr = __low2half(p);
+    *pb = __high2half(p);
+  }
+};
+template <>
+struct Pair<StBF16> {
+  using T = __nv_bfloat16;
+  static __device__ __forceinline__ float2 cv(T r, T b, float w) {
+    return vadd(make_float2(w, w), make_float2(__bfloat162float(r), __bfloat162float(b)));
+  }
+  static __device__ __forceinline__ void st(T* pr, T* pb, float2 v, float w) {
+    const float2 h = vsub(v, make_float2(w, w));
+    const __nv_bfloat162 p = __floats2bfloat162_rn(h.x, h.y);
+    *pr = __low2bfloat16(p);
+    *pb = __high2bfloat16(p);
   }
 };
 
@@ -248,15 +366,14 @@ struct PullIdx {
 
 template <class S>
 __device__ __forceinline__ void pull_full(const LatDev& L, const typename S::T* __restrict__ src, const PullIdx& P,
-                                          float (&fr)[Q], float (&fb)[Q]) {
+                                          float2 (&f)[Q]) {
   const long long cstride = (long long)Q * L.np;
   Unroll<0, Q>::run([&](auto ic) {
     constexpr int I = decltype(ic)::value;
     int idx, d;
     P.template at<I>(idx, d);
     const typename S::T* p = src + (long long)d * L.np + idx;
-    fr[I] = S::ld(p, wgt(I));
-    fb[I] = S::ld(p + cstride, wgt(I));
+    f[I] = make_float2(S::ld(p, wgt(I)), S::ld(p + cstride, wgt(I)));
   });
 }
 
@@ -280,44 +397,45 @@ __device__ __forceinline__ uint32_t pull_async(const LatDev& L, const typename S
 
 // Density from the 19 populations of a site: opposite pairs (I, I+1) first, then
 // a balanced tree (depth 5, so the additions overlap), in one fixed order that
-// every kernel uses; get(i) yields population i, so values can be summed as they
-// are loaded.
-template <class Get>
-__device__ __forceinline__ float sum19_of(Get&& get) {
+// every kernel uses; get(i) yields population i (a float or a pair), so values can be
+// summed as they are loaded.
+template <class V, class Get>
+__device__ __forceinline__ V sum19_of(Get&& get) {
   auto pair = [&](auto ic) {
     constexpr int I = 1 + 2 * decltype(ic)::value;
-    return __fadd_rn(get(std::integral_constant<int, I>()), get(std::integral_constant<int, I + 1>()));
+    return vadd(get(std::integral_constant<int, I>()), get(std::integral_constant<int, I + 1>()));
   };
   using std::integral_constant;
-  const float c0 = __fadd_rn(pair(integral_constant<int, 0>()), pair(integral_constant<int, 1>()));
-  const float c1 = __fadd_rn(pair(integral_constant<int, 2>()), pair(integral_constant<int, 3>()));
-  const float c2 = __fadd_rn(pair(integral_constant<int, 4>()), pair(integral_constant<int, 5>()));
-  const float c3 = __fadd_rn(pair(integral_constant<int, 6>()), pair(integral_constant<int, 7>()));
-  const float c4 = __fadd_rn(pair(integral_constant<int, 8>()), get(integral_constant<int, 0>()));
-  return __fadd_rn(__fadd_rn(__fadd_rn(c0, c1), __fadd_rn(c2, c3)), c4);
+  const V c0 = vadd(pair(integral_constant<int, 0>()), pair(integral_constant<int, 1>()));
+  const V c1 = vadd(pair(integral_constant<int, 2>()), pair(integral_constant<int, 3>()));
+  const V c2 = vadd(pair(integral_constant<int, 4>()), pair(integral_constant<int, 5>()));
+  const V c3 = vadd(pair(integral_constant<int, 6>()), pair(integral_constant<int, 7>()));
+  const V c4 = vadd(pair(integral_constant<int, 8>()), get(integral_constant<int, 0>()));
+  return vadd(vadd(vadd(c0, c1), vadd(c2, c3)), c4);
 }
-__device__ __forceinline__ float sum19(const float (&f)[Q]) {
-  return sum19_of([&](auto ic) { return f[decltype(ic)::value]; });
+template <class V>
+__device__ __forceinline__ V sum19(const V (&f)[Q]) {
+  return sum19_of<V>([&](auto ic) { return f[decltype(ic)::value]; });
 }
 
 // Evaporation boundary (Sec. II C) on the densities of the arrived populations:
 // rho^r := rho_H, rho^b := rho^r + rho^b - rho_H.
-__device__ __forceinline__ void sink_densities(const LatDev& L, float& rr, float& rb) {
-  const float rbn = (rr + rb) - L.rhoH;
-  rr = L.rhoH;
-  rb = rbn;
+__device__ __forceinline__ void sink_densities(const LatDev& L, float2& rho) {
+  rho.y = __fsub_rn(__fadd_rn(rho.x, rho.y), L.rhoH);
+  rho.x = L.rhoH;
 }
 
 // Reset value of direction i for density rho (f^eq at rest), an exact float product.
-__device__ __forceinline__ float rest_pop(int i, float rho) { return __fmul_rn(wgt(i), rho); }
+template <class V>
+__device__ __forceinline__ V rest_pop(int i, V rho) { return vmul(vset<V>(wgt(i)), rho); }
 
 // Evaporated mass of one sink site: sum_i (f_i^r - w_i rho_H) over the arrived r
 // populations, without contraction, so that where only reset values arrived (inside
 // the sink region) every term is exactly zero and no rounding bias is booked.
-__device__ __forceinline__ float sink_excess(const LatDev& L, const float (&fr)[Q]) {
+__device__ __forceinline__ float sink_excess(const LatDev& L, const float2 (&f)[Q]) {
   float e = 0.0f;
 #pragma unroll
-  for (int i = 0; i < Q; ++i) e = __fadd_rn(e, __fsub_rn(fr[i], rest_pop(i, L.rhoH)));
+  for (int i = 0; i < Q; ++i) e = __fadd_rn(e, __fsub_rn(f[i].x, rest_pop(i, L.rhoH)));
   return e;
 }
 
@@ -332,27 +450,27 @@ __device__ __forceinline__ float psi_of(float rho) {
   }
   return 1.0f - expf(-rho);
 }
+__device__ __forceinline__ float2 psi_of(float2 rho) { return make_float2(psi_of(rho.x), psi_of(rho.y)); }
 
 template <class S>
 __device__ __forceinline__ void store_site(const LatDev& L, typename S::T* __restrict__ dst, int s,
-                                           const float (&fr)[Q], const float (&fb)[Q]) {
+                                           const float2 (&f)[Q]) {
   const long long cstride = (long long)Q * L.np;
 #pragma unroll
   for (int i = 0; i < Q; ++i) {
     typename S::T* p = dst + (long long)i * L.np + s;
-    S::st(p, fr[i], wgt(i));
-    S::st(p + cstride, fb[i], wgt(i));
+    Pair<S>::st(p, p + cstride, f[i], wgt(i));
   }
 }
 
-// Momentum sum_i f_i e_i of one component.
-// Momentum sum_i f_i e_i of one component from the differences of opposite
+// Momentum sum_i f_i e_i of each component from the differences of opposite
 // pairs, d = f_I - f_{I+1} (e_{I+1} = -e_I): each axis sums the five d whose
 // e_I has a component along it.
-__device__ __forceinline__ void momentum(const float (&f)[Q], float (&m)[3]) {
-  float d[9];
+template <class V>
+__device__ __forceinline__ void momentum(const V (&f)[Q], V (&m)[3]) {
+  V d[9];
 #pragma unroll
-  for (int k = 0; k < 9; ++k) d[k] = __fsub_rn(f[1 + 2 * k], f[2 + 2 * k]);
+  for (int k = 0; k < 9; ++k) d[k] = vsub(f[1 + 2 * k], f[2 + 2 * k]);
   bool first[3] = {true, true, true};
   Unroll<0, 9>::run([&](auto kc) {
     constexpr int K = decltype(kc)::value, I = 1 + 2 * K;
@@ -360,143 +478,117 @@ __device__ __forceinline__ void momentum(const float (&f)[Q], float (&m)[3]) {
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
       if (e[a] == 0) continue;
-      if (first[a]) m[a] = e[a] > 0 ? d[K] : -d[K];
-      else m[a] = e[a] > 0 ? __fadd_rn(m[a], d[K]) : __fsub_rn(m[a], d[K]);
+      if (first[a]) m[a] = e[a] > 0 ? d[K] : vneg(d[K]);
+      else m[a] = e[a] > 0 ? vadd(m[a], d[K]) : vsub(m[a], d[K]);
       first[a] = false;
     }
   });
 }
 
-// The collision arithmetic below spells out every rounding (__fmul_rn, __fmaf_rn,
-// ...) so that the compiler cannot contract it differently in different kernels:
+// The collision arithmetic below spells out every rounding (vmul, vfma, ...) so that the compiler cannot contract it differently in different kernels:
 // every step kernel produces the same bits for the same state.
 
 // Common velocity u' = sum_c (m^c / tau_c) / sum_c (rho^c / tau_c) (Sec. II A: the
 // mass-weighted u_eq when tau_r = tau_b).
-__device__ __forceinline__ void common_velocity(const LatDev& L, float rr, float rb, const float (&mr)[3],
-                                                const float (&mb)[3], float (&up)[3]) {
+__device__ __forceinline__ void common_velocity(const LatDev& L, float2 rho, const float2 (&m)[3], float (&up)[3]) {
   const float omr = L.omega[0], omb = L.omega[1];
-  const float den = __fmaf_rn(rr, omr, __fmul_rn(rb, omb));
+  const float den = __fmaf_rn(rho.x, omr, __fmul_rn(rho.y, omb));
   const float inv = den > 0.0f ? __fdiv_rn(1.0f, den) : 0.0f;
 #pragma unroll
-  for (int d = 0; d < 3; ++d) up[d] = __fmul_rn(__fmaf_rn(mr[d], omr, __fmul_rn(mb[d], omb)), inv);
+  for (int d = 0; d < 3; ++d) up[d] = __fmul_rn(__fmaf_rn(m[d].x, omr, __fmul_rn(m[d].y, omb)), inv);
 }
 
 // c . u for a D3Q19 direction, summing the non-zero terms in x, y, z order.
-template <int I>
-__device__ __forceinline__ float cdot(const float (&u)[3]) {
+template <int I, class V>
+__device__ __forceinline__ V cdot(const V (&u)[3]) {
   constexpr int ex = dir_x(I), ey = dir_y(I), ez = dir_z(I);
-  float r = 0.0f;
+  V r = vset<V>(0.0f);
   bool first = true;
-  if (ex != 0) { r = ex > 0 ? u[0] : -u[0]; first = false; }
-  if (ey != 0) { r = first ? (ey > 0 ? u[1] : -u[1]) : (ey > 0 ? __fadd_rn(r, u[1]) : __fsub_rn(r, u[1])); first = false; }
-  if (ez != 0) { r = first ? (ez > 0 ? u[2] : -u[2]) : (ez > 0 ? __fadd_rn(r, u[2]) : __fsub_rn(r, u[2])); }
+  if (ex != 0) { r = ex > 0 ? u[0] : vneg(u[0]); first = false; }
+  if (ey != 0) { r = first ? (ey > 0 ? u[1] : vneg(u[1])) : (ey > 0 ? vadd(r, u[1]) : vsub(r, u[1])); first = false; }
+  if (ez != 0) { r = first ? (ez > 0 ? u[2] : vneg(u[2])) : (ez > 0 ? vadd(r, u[2]) : vsub(r, u[2])); }
   return r;
 }
 
-// Shifted-velocity BGK relaxation of component c at a fluid site (Eqs. (1)-(3)):
-// u_eq = u' + tau_c F^c / rho^c with F^c = -Psi^c(x) g A: g = G and A = a^cbar =
-// sum_i w_i Psi^cbar(x + e_i) e_i in the paper's two-component model, g = 1 and
-// A = sum_cbar g^{c cbar} a^cbar (coupled_sums) with self couplings.
-__device__ __forceinline__ void relax_core(float om, float tau, float (&f)[Q], float rho, float ps, float g,
-                                           const float (&A)[3], const float (&up)[3]) {
+// -g tau Psi / rho, the factor of A in the velocity shift (relax_core).
+__device__ __forceinline__ float shift_factor(float g, float tau, float rho, float ps) {
+  const float q = rho > 0.0f ? __fdiv_rn(ps, rho) : 0.0f;
+  return __fmul_rn(__fmul_rn(-g, tau), q);
+}
+__device__ __forceinline__ float2 shift_factor(float2 g, float2 tau, float2 rho, float2 ps) {
+  return make_float2(shift_factor(g.x, tau.x, rho.x, ps.x), shift_factor(g.y, tau.y, rho.y, ps.y));
+}
+
+// Shifted-velocity BGK relaxation of a component (V = float) or of both (float2) at a
+// fluid site (Eqs. (1)-(3)): u_eq = u' + tau_c F^c / rho^c with F^c = -Psi^c(x) g A: g = G
+// and A = a^cbar = sum_i w_i Psi^cbar(x + e_i) e_i in the paper's two-component model,
+// g = 1 and A = sum_cbar g^{c cbar} a^cbar (coupled_sums) with self couplings.
+template <class V>
+__device__ __forceinline__ void relax_core(V om, V tau, V (&f)[Q], V rho, V ps, V g, const V (&A)[3],
+                                           const float (&up)[3]) {
   // tau F / rho = (-g tau) (Psi / rho) A with Psi / rho <= 1, so a trace (or
   // denormal) density cannot overflow the shift; rho = 0 takes u' itself
-  const float q = rho > 0.0f ? __fdiv_rn(ps, rho) : 0.0f;
-  const float gq = __fmul_rn(__fmul_rn(-g, tau), q);
-  float u[3];
+  const V gq = shift_factor(g, tau, rho, ps);
+  V u[3];
 #pragma unroll
-  for (int d = 0; d < 3; ++d) u[d] = __fmaf_rn(gq, A[d], up[d]);
-  const float usq = __fmaf_rn(u[0], u[0], __fmaf_rn(u[1], u[1], __fmul_rn(u[2], u[2])));
-  const float base = __fmaf_rn(-1.5f, usq, 1.0f);  // 1 - 1.5 u.u
+  for (int d = 0; d < 3; ++d) u[d] = vfma(gq, A[d], vset<V>(up[d]));
+  const V usq = vfma(u[0], u[0], vfma(u[1], u[1], vmul(u[2], u[2])));
+  const V base = vfma(vset<V>(-1.5f), usq, vset<V>(1.0f));  // 1 - 1.5 u.u
   // f^eq_i = w_i rho (1 + 3 c.u + 4.5 (c.u)^2 - 1.5 u.u); opposite directions share
   // the even part w rho (1 - 1.5 u.u) + 4.5 w rho (c.u)^2 and differ in the sign of
   // the odd part 3 w rho c.u. The factors of w rho are formed once per weight class.
-  f[0] = __fmaf_rn(om, __fsub_rn(__fmul_rn(__fmul_rn(kW0, rho), base), f[0]), f[0]);
-  const float wr1 = __fmul_rn(kW1, rho), wr2 = __fmul_rn(kW2, rho);
-  const float wb1 = __fmul_rn(wr1, base), wb2 = __fmul_rn(wr2, base);
-  const float w451 = __fmul_rn(4.5f, wr1), w452 = __fmul_rn(4.5f, wr2);
-  const float w31 = __fmul_rn(3.0f, wr1), w32 = __fmul_rn(3.0f, wr2);
+  f[0] = vfma(om, vsub(vmul(vmul(vset<V>(kW0), rho), base), f[0]), f[0]);
+  const V wr1 = vmul(vset<V>(kW1), rho), wr2 = vmul(vset<V>(kW2), rho);
+  const V wb1 = vmul(wr1, base), wb2 = vmul(wr2, base);
+  const V w451 = vmul(vset<V>(4.5f), wr1), w452 = vmul(vset<V>(4.5f), wr2);
+  const V w31 = vmul(vset<V>(3.0f), wr1), w32 = vmul(vset<V>(3.0f), wr2);
   Unroll<0, 9>::run([&](auto kc) {
     constexpr int I = 1 + 2 * decltype(kc)::value, J = I + 1;
     constexpr bool axis = I <= 6;
-    const float cu = cdot<I>(u);
-    const float ev = __fmaf_rn(__fmul_rn(axis ? w451 : w452, cu), cu, axis ? wb1 : wb2);
-    const float od = __fmul_rn(axis ? w31 : w32, cu);
-    f[I] = __fmaf_rn(om, __fsub_rn(__fadd_rn(ev, od), f[I]), f[I]);
-    f[J] = __fmaf_rn(om, __fsub_rn(__fsub_rn(ev, od), f[J]), f[J]);
+    const V cu = cdot<I>(u);
+    const V ev = vfma(vmul(axis ? w451 : w452, cu), cu, axis ? wb1 : wb2);
+    const V od = vmul(axis ? w31 : w32, cu);
+    f[I] = vfma(om, vsub(vadd(ev, od), f[I]), f[I]);
+    f[J] = vfma(om, vsub(vsub(ev, od), f[J]), f[J]);
   });
 }
-__device__ __forceinline__ void relax(const LatDev& L, int c, float (&f)[Q], float rho, float ps, float g,
-                                      const float (&A)[3], const float (&up)[3]) {
-  relax_core(c == 0 ? L.omega[0] : L.omega[1], c == 0 ? L.tau[0] : L.tau[1], f, rho, ps, g, A, up);
-}
 
-// A^c = sum_cbar g^{c cbar} a^cbar of Eq. (3): the cross coupling g (= g^{rb} = g^{br})
-// times the other component's sum, plus the self coupling g^{cc} times its own
-// (an exact zero when g^{cc} = 0, the paper's two-component model).
-__device__ __forceinline__ void coupled_sums(const LatDev& L, const float (&ar)[3], const float (&ab)[3],
-                                             float (&Ar)[3], float (&Ab)[3]) {
-#pragma unroll
-  for (int d = 0; d < 3; ++d) {
-    Ar[d] = __fmaf_rn(L.Gs[0], ar[d], __fmul_rn(L.G, ab[d]));
-    Ab[d] = __fmaf_rn(L.Gs[1], ab[d], __fmul_rn(L.G, ar[d]));
-  }
-}
-
-// Shifted-velocity BGK collision of one fluid site, in place on fr/fb.
-// ar/ab: sum_i w_i Psi^{r|b}(x + e_i) e_i.
-__device__ __forceinline__ void collide(const LatDev& L, float (&fr)[Q], float (&fb)[Q], float rr, float rb, float psr,
-                                        float psb, const float (&ar)[3], const float (&ab)[3]) {
-  float mr[3], mb[3], up[3];
-  momentum(fr, mr);
-  momentum(fb, mb);
-  common_velocity(L, rr, rb, mr, mb, up);
+// Shifted-velocity BGK collision of one fluid site, in place on f. a[d] holds the sums
+// (a^r, a^b) = sum_i w_i Psi^{r|b}(x + e_i) e_i. A^c = sum_cbar g^{c cbar} a^cbar of
+// Eq. (3): the cross coupling g (= g^{rb} = g^{br}) times the other component's sum, plus
+// the self coupling g^{cc} times its own.
+__device__ __forceinline__ void collide(const LatDev& L, float2 (&f)[Q], float2 rho, float2 ps, const float2 (&a)[3]) {
+  float2 m[3], A[3], g;
+  float up[3];
+  momentum(f, m);
+  common_velocity(L, rho, m, up);
   if (L.Gs[0] == 0.0f && L.Gs[1] == 0.0f) {  // the paper's model: the cross coupling alone
-    relax(L, 0, fr, rr, psr, L.G, ab, up);
-    relax(L, 1, fb, rb, psb, L.G, ar, up);
+    g = make_float2(L.G, L.G);
+#pragma unroll
+    for (int d = 0; d < 3; ++d) A[d] = make_float2(a[d].y, a[d].x);
   } else {
-    float Ar[3], Ab[3];
-    coupled_sums(L, ar, ab, Ar, Ab);
-    relax(L, 0, fr, rr, psr, 1.0f, Ar, up);
-    relax(L, 1, fb, rb, psb, 1.0f, Ab, up);
+    g = make_float2(1.0f, 1.0f);
+#pragma unroll
+    for (int d = 0; d < 3; ++d)
+      A[d] = make_float2(__fmaf_rn(L.Gs[0], a[d].x, __fmul_rn(L.G, a[d].y)),
+                         __fmaf_rn(L.Gs[1], a[d].y, __fmul_rn(L.G, a[d].x)));
   }
+  relax_core(make_float2(L.omega[0], L.omega[1]), make_float2(L.tau[0], L.tau[1]), f, rho, ps, g, A, up);
 }
 
-// sum_i w_i Psi^c(x + e_i) e_i of both components from a Psi ring whose cells hold
-// (Psi^r, Psi^b); psi2(plane slot, ly, lx). Opposite pairs (I, I+1) contribute
-// w_I (Psi(x + e_I) - Psi(x - e_I)) e_I.
-template <class PsiAt2>
-__device__ __forceinline__ void force_sums(PsiAt2 psi2, int sm1, int s0, int sp1, int ly, int lx, float (&ar)[3],
-                                           float (&ab)[3]) {
-  ar[0] = ar[1] = ar[2] = 0.f;
-  ab[0] = ab[1] = ab[2] = 0.f;
+// sum_i w_i Psi^c(x + e_i) e_i from a Psi ring: of both components (V = float2, cells
+// (Psi^r, Psi^b)) or of one (float); psi(plane slot, ly, lx). Opposite pairs (I, I+1)
+// contribute w_I (Psi(x + e_I) - Psi(x - e_I)) e_I.
+template <class V, class PsiAt>
+__device__ __forceinline__ void force_sums(PsiAt psi, int sm1, int s0, int sp1, int ly, int lx, V (&a)[3]) {
+  a[0] = a[1] = a[2] = vset<V>(0.f);
   Unroll<0, 9>::run([&](auto kc) {
     constexpr int I = 1 + 2 * decltype(kc)::value;
     constexpr int ex = dir_x(I), ey = dir_y(I), ez = dir_z(I);
     const int sa = ez > 0 ? sp1 : (ez < 0 ? sm1 : s0);
     const int sb = ez > 0 ? sm1 : (ez < 0 ? sp1 : s0);
-    const float2 pa = psi2(sa, ly + ey, lx + ex), pb = psi2(sb, ly - ey, lx - ex);
-    const float dr = __fsub_rn(pa.x, pb.x), db = __fsub_rn(pa.y, pb.y);
-    auto acc = [&](float& a, int e, float d) { a = __fmaf_rn(e > 0 ? wgt(I) : -wgt(I), d, a); };
-    if (ex != 0) { acc(ar[0], ex, dr); acc(ab[0], ex, db); }
-    if (ey != 0) { acc(ar[1], ey, dr); acc(ab[1], ey, db); }
-    if (ez != 0) { acc(ar[2], ez, dr); acc(ab[2], ez, db); }
-  });
-}
-
-// sum_i w_i Psi(x + e_i) e_i of one component, with force_sums' order of operations;
-// psi1(plane slot, ly, lx) yields that component's Psi.
-template <class PsiAt1>
-__device__ __forceinline__ void force_sum_one(PsiAt1 psi1, int sm1, int s0, int sp1, int ly, int lx, float (&a)[3]) {
-  a[0] = a[1] = a[2] = 0.f;
-  Unroll<0, 9>::run([&](auto kc) {
-    constexpr int I = 1 + 2 * decltype(kc)::value;
-    constexpr int ex = dir_x(I), ey = dir_y(I), ez = dir_z(I);
-    const int sa = ez > 0 ? sp1 : (ez < 0 ? sm1 : s0);
-    const int sb = ez > 0 ? sm1 : (ez < 0 ? sp1 : s0);
-    const float d = __fsub_rn(psi1(sa, ly + ey, lx + ex), psi1(sb, ly - ey, lx - ex));
-    auto acc = [&](float& v, int e) { v = __fmaf_rn(e > 0 ? wgt(I) : -wgt(I), d, v); };
+    const V d = vsub(psi(sa, ly + ey, lx + ex), psi(sb, ly - ey, lx - ex));
+    auto acc = [&](V& v, int e) { v = vfma(vset<V>(e > 0 ? wgt(I) : -wgt(I)), d, v); };
     if (ex != 0) acc(a[0], ex);
     if (ey != 0) acc(a[1], ey);
     if (ez != 0) acc(a[2], ez);
@@ -543,7 +635,8 @@ struct Tile {
   bool active, has_halo;
   double evap;
 
-  __device__ __forceinline__ Tile(const LatDev& L_, Smem& sm_, const typename S::T* s_, typename S::T* d_)
+  __device__ __forceinline__ Tile(const LatDev& L_, Smem& sm_, const typename S::T* s_, typename S::T* d_,
+                                  const CUtensorMap* = nullptr)
       : L(L_), sm(sm_), src(s_), dst(d_), evap(0.0) {}
 
   __device__ __forceinline__ int wrapz(int z) const { return z < 0 ? z + L.nz : (z >= L.nz ? z - L.nz : z); }
@@ -583,70 +676,62 @@ struct Tile {
     cp_async_commit();
   }
 
-  // Read plane p out of the slots (after the wait): the own site into fr/fb, the
+  // Read plane p out of the slots (after the wait): the own site into f, the
   // halo site as sums; apply the sink and publish Psi to ring slot p & 3.
-  __device__ __forceinline__ void take(int p, bool own, int cls, uint32_t hi, int hcl, uint32_t hhi,
-                                       float (&fr)[Q], float (&fb)[Q], float& rr, float& rb) {
+  __device__ __forceinline__ void take(int p, bool own, int cls, uint32_t hi, int hcl, uint32_t hhi, float2 (&f)[Q],
+                                       float2& rho) {
     const int slot = p & 3;
-    float pr = 0.0f, pb = 0.0f;
+    float2 ps = make_float2(0.0f, 0.0f);
     if (cls == SOLID) {
-      rr = rb = 0.0f;
+      rho = ps;
     } else {
       const uint32_t* w = own_slot();
 #pragma unroll
       for (int i = 0; i < Q; ++i) {
         const uint32_t h = (hi >> i) & 1u;
-        fr[i] = S::word(w[i * NT], h, wgt(i));
-        fb[i] = S::word(w[(Q + i) * NT], h, wgt(i));
+        f[i] = make_float2(S::word(w[i * NT], h, wgt(i)), S::word(w[(Q + i) * NT], h, wgt(i)));
       }
-      rr = sum19(fr);
-      rb = sum19(fb);
+      rho = sum19(f);
       if (cls == SINK) {
-        if (active && own && own_z(L, wrapz(p))) evap += (double)sink_excess(L, fr);
-        sink_densities(L, rr, rb);
+        if (active && own && own_z(L, wrapz(p))) evap += (double)sink_excess(L, f);
+        sink_densities(L, rho);
       }
-      pr = psi_of(rr);
-      pb = psi_of(rb);
+      ps = psi_of(rho);
     }
-    sm.ring[slot][ty + 1][tx + 1] = make_float2(pr, pb);
+    sm.ring[slot][ty + 1][tx + 1] = ps;
     if (has_halo) {
-      float hpr = 0.0f, hpb = 0.0f;
+      float2 hps = make_float2(0.0f, 0.0f);
       if (hcl != SOLID) {
         const uint32_t* w = halo_slot();
         // the owner's arithmetic, so the halo Psi has the owner's bits
-        float hrr = sum19_of([&](auto ic) {
+        float2 hrho = sum19_of<float2>([&](auto ic) {
           constexpr int I = decltype(ic)::value;
-          return S::word(w[I * HS], (hhi >> I) & 1u, wgt(I));
+          const uint32_t h = (hhi >> I) & 1u;
+          return make_float2(S::word(w[I * HS], h, wgt(I)), S::word(w[(Q + I) * HS], h, wgt(I)));
         });
-        float hrb = sum19_of([&](auto ic) {
-          constexpr int I = decltype(ic)::value;
-          return S::word(w[(Q + I) * HS], (hhi >> I) & 1u, wgt(I));
-        });
-        if (hcl == SINK) sink_densities(L, hrr, hrb);
-        hpr = psi_of(hrr);
-        hpb = psi_of(hrb);
+        if (hcl == SINK) sink_densities(L, hrho);
+        hps = psi_of(hrho);
       }
-      sm.ring[slot][hly + 1][hlx + 1] = make_float2(hpr, hpb);
+      sm.ring[slot][hly + 1][hlx + 1] = hps;
     }
   }
 
   // Collide plane z (in [0, nz); read out one plane earlier) and store f*.
-  __device__ __forceinline__ void finish(int z, float (&fr)[Q], float (&fb)[Q], float rr, float rb, int cls) {
+  __device__ __forceinline__ void finish(int z, float2 (&f)[Q], float2 rho, int cls) {
     if (!active || cls == SOLID) return;
     const int s = x + L.nx * y + L.nxny * z;
     if (cls == SINK) {
       // Sinks are neither forced nor collided: they stream f^eq(rho_H, 0) and
       // f^eq(rho^r + rho^b - rho_H, 0) as they are.
 #pragma unroll
-      for (int i = 0; i < Q; ++i) { fr[i] = rest_pop(i, rr); fb[i] = rest_pop(i, rb); }
+      for (int i = 0; i < Q; ++i) f[i] = rest_pop(i, rho);
     } else {
-      float ar[3], ab[3];
-      auto psi2 = [&](int sl, int ly, int lx) { return sm.ring[sl][ly + 1][lx + 1]; };
-      force_sums(psi2, (z - 1) & 3, z & 3, (z + 1) & 3, ty, tx, ar, ab);
-      const float2 ps = sm.ring[z & 3][ty + 1][tx + 1];
-      collide(L, fr, fb, rr, rb, ps.x, ps.y, ar, ab);
+      float2 a[3];
+      auto psi = [&](int sl, int ly, int lx) { return sm.ring[sl][ly + 1][lx + 1]; };
+      force_sums(psi, (z - 1) & 3, z & 3, (z + 1) & 3, ty, tx, a);
+      collide(L, f, rho, sm.ring[z & 3][ty + 1][tx + 1], a);
     }
-    store_site<S>(L, dst, s, fr, fb);
+    store_site<S>(L, dst, s, f);
   }
 
   // March planes [zb, ze) upward (down = false) or downward. Plane p is read out
@@ -654,9 +739,9 @@ struct Tile {
   // barrier plane p - d (whose Psi neighbours are now all in the ring) collides.
   // The halo plane on each end is staged for Psi only. The ring slot of plane
   // p is p & 3 for p = -1 too, as in finish().
-  __device__ __forceinline__ void run(int zb, int ze, bool down) {
-    float cr[Q], cb[Q], nr[Q], nb[Q];
-    float crr = 0.f, crb = 0.f, nrr = 0.f, nrb = 0.f;
+  __device__ __forceinline__ bool run(int zb, int ze, bool down) {
+    float2 c[Q], n2[Q];
+    float2 crho = make_float2(0.f, 0.f), nrho = crho;
     int ccl = SOLID, ncl = SOLID, hcl = SOLID;
     uint32_t hi = 0u, hhi = 0u;
     const int d = down ? -1 : 1;
@@ -666,17 +751,17 @@ struct Tile {
     for (int o = 0; o < n + 2; ++o) {
       const int p = first + (o - 1) * d;
       cp_async_wait_all();
-      take(p, o >= 1 && o <= n, ncl, hi, hcl, hhi, nr, nb, nrr, nrb);
+      take(p, o >= 1 && o <= n, ncl, hi, hcl, hhi, n2, nrho);
       const int pcl = ncl;
       if (o + 1 < n + 2) issue(p + d, ncl, hi, hcl, hhi);
       __syncthreads();
-      if (o >= 2) finish(p - d, cr, cb, crr, crb, ccl);
+      if (o >= 2) finish(p - d, c, crho, ccl);
 #pragma unroll
-      for (int i = 0; i < Q; ++i) { cr[i] = nr[i]; cb[i] = nb[i]; }
-      crr = nrr;
-      crb = nrb;
+      for (int i = 0; i < Q; ++i) c[i] = n2[i];
+      crho = nrho;
       ccl = pcl;
     }
+    return true;
   }
 
   // Block sum of the evaporated mass (fixed order: warps, then warp 0's lanes).
@@ -696,52 +781,71 @@ struct Tile {
 
 // ------------------------------------------------------------------ fused step, staged rows
 //
-// The same march as Tile, with the pulls staged cooperatively. For each of the
-// 38 (component, direction) pairs the plane's source rows -- the TY + 2 rows
-// y0 - 1 .. y0 + TY shifted by -e_y, in plane z - e_z -- are copied into shared
-// memory over columns x0 - E .. x0 + TX + E as aligned 16-byte chunks (E
-// populations each), and the x shift -e_x is applied when a thread reads them.
-// The E-column margins hold the side halo, so the halo needs no pulls of its
-// own. Chunks are spread evenly over the CTA's threads (a per-plane table holds
-// each row's offset, a per-column table each chunk's wrapped x), so no warp
-// carries more copy work than another. Requires nx % E == 0 (then every
-// wrapped chunk is aligned). A population whose source plane is solid is the
+// The same march as Tile, with the pulls staged cooperatively. For each of the 19
+// directions the plane's source rows -- the TY + 2 rows y0 - 1 .. y0 + TY shifted by
+// -e_y, in plane z - e_z -- are copied into shared memory over columns x0 - E ..
+// x0 + TX + E (E populations are 16 bytes), and the x shift -e_x is applied when a thread
+// reads them. The E-column margins hold the side halo, so the halo needs no pulls of its
+// own. One direction is one TMA box of both components. Requires nx % E == 0 (then the
+// box starts on a 16-byte boundary). A population whose source plane is solid is the
 // site's own opposite population (halfway bounce-back): read directly.
 //
-// Per plane: wait for the copies, barrier, read out plane p (Psi to the ring,
-// own populations to registers), write the row table of plane p + d, barrier,
-// start plane p + d's copies, collide plane p - d.
+// TMA fills what lies outside the lattice with zeros, so each thread also fetches its
+// share of 16-byte pieces with cp.async into a side buffer -- the left margin of the
+// first tile in x, the right margin of every other one, and at the y edges the outermost
+// rows, all periodic -- and moves them into the staged rows once the boxes have landed.
+// Only the last right margin needs that; the others fetch theirs so that all tiles take
+// the same time: with the pieces at lattice edges alone, edge tiles ran 10% slower, fell
+// planes behind their neighbours, and the rows and 128-byte lines that neighbours share
+// were read from DRAM again (512^3 FP32, 64 x 4 tiles: 47 GB read per step against 23.7 GB,
+// 10.75 ms against 7.2 ms).
+//
+// Per plane: wait for the copies, read out plane p (Psi to the ring, own populations
+// to registers), barrier, start plane p + d's copies, collide plane p - d.
 template <int TX, int TY, class S>
 struct TileRows {
   using T = typename S::T;
-  static constexpr int E = 16 / (int)sizeof(T);           // populations per chunk
+  static constexpr int E = 16 / (int)sizeof(T);           // populations per 16 bytes
   static constexpr int NT = TX * TY, NW = NT / 32, RW = TX + 2, RH = TY + 2, NH = 2 * TX + 2 * RH;
   static constexpr int SW = TX + 2 * E;                   // staged row width
-  static constexpr int CH = SW / E;                       // chunks per row
+  static constexpr int CH = SW / E;                       // 16-byte pieces per staged row
   static constexpr int NR = 2 * Q * RH;                   // staged rows per plane
-  static constexpr int RS = NT / CH;                      // rows copied per pass of the CTA
+  static constexpr int BOX = 2 * RH * SW;                 // populations per box
+  static constexpr int IS = (BOX * (int)sizeof(T) + 127) / 128 * 128 / (int)sizeof(T);  // box stride (128-byte aligned)
+  static constexpr int YR = 38;                           // wrapped rows per y edge: 2 (5 directions x 2 + 9 x 1)
   static_assert(TX % E == 0, "tile width must be a multiple of the chunk");
   static_assert(NH <= NT && NT % 32 == 0, "tile shape");
 
   struct Smem {
-    T stage[2 * Q][RH][SW];  // rows of plane p: [c Q + i][y - y0 + 1][x - x0 + E]
+    T stage[Q * IS];         // rows of plane p: [i][c][y - y0 + 1][x - x0 + E], box i at i IS
     float2 ring[4][RH][RW];  // (Psi^r, Psi^b) of plane slot, tile row + 1, tile column + 1
-    const T* rowp[NR];       // source address of each staged row's column x = 0
-    int chx[CH];             // wrapped x of chunk j
     double red[NW];
+    uint64_t bar;            // completes when a plane's boxes have landed
+    alignas(16) T side[1];   // wrapped pieces: x edges [edge][row][E], then y edges [edge][row][SW]
   };
+  // Bytes of shared memory for xe sides in x and ye edges in y of one tile (1, or 2 where
+  // one tile spans the lattice).
+  static constexpr size_t smem_bytes(int xe, int ye) {
+    return sizeof(Smem) + sizeof(T) * ((size_t)xe * NR * E + (size_t)ye * YR * SW);
+  }
 
   const LatDev& L;
   Smem& sm;
   const T* __restrict__ src;
   T* __restrict__ dst;
-  int tx, ty, x, y, hx, hy, hlx, hly, y0;
-  int cr0, cj;  // this thread's copy work: rows cr0, cr0 + RS, ... at chunk cj (cr0 >= NR: none)
+  const CUtensorMap* map;
+  int tx, ty, x, y, hx, hy, hlx, hly, x0, y0;
+  int tw, th;                  // the tile's sites in x and y
+  bool left, right, low, high; // margins and edge rows that come through the side buffer
+  unsigned parity;             // of the plane in flight
   bool active, has_halo;
   double evap;
 
-  __device__ __forceinline__ TileRows(const LatDev& L_, Smem& sm_, const T* s_, T* d_)
-      : L(L_), sm(sm_), src(s_), dst(d_), evap(0.0) {}
+  __device__ __forceinline__ TileRows(const LatDev& L_, Smem& sm_, const T* s_, T* d_, const CUtensorMap* m_)
+      : L(L_), sm(sm_), src(s_), dst(d_), map(m_), parity(0), evap(0.0) {
+    if (threadIdx.x == 0) mbar_init(&sm.bar, 1);
+    __syncthreads();
+  }
 
   __device__ __forceinline__ int wrapz(int z) const { return z < 0 ? z + L.nz : (z >= L.nz ? z - L.nz : z); }
 
@@ -753,7 +857,14 @@ struct TileRows {
     active = gx < L.nx && gy < L.ny;
     x = gx % L.nx;
     y = gy % L.ny;
+    x0 = bx * TX;
     y0 = by * TY;
+    tw = min(TX, L.nx - x0);
+    th = min(TY, L.ny - y0);
+    left = x0 == 0;
+    right = !left || x0 + TX >= L.nx;
+    low = y0 < 2;
+    high = y0 + TY + 2 > L.ny;
     const int h = tid;  // halo slot: top row, bottom row, left column, right column
     has_halo = h < NH;
     if (h < TX) { hlx = h; hly = -1; }
@@ -762,153 +873,200 @@ struct TileRows {
     else { hlx = TX; hly = h - 2 * TX - RH - 1; }
     hx = wrapi(bx * TX + hlx, L.nx);
     hy = wrapi(by * TY + hly, L.ny);
-    if (tid < CH) sm.chx[tid] = wrapi(bx * TX - E + tid * E, L.nx);
-    cj = tid % CH;
-    cr0 = tid < RS * CH ? tid / CH : NR;
   }
 
-  // Row table of plane p (p in [-1, nz]).
-  __device__ __forceinline__ void table(int p) {
-    const int zp = wrapz(p);
-    for (int R = threadIdx.x; R < NR; R += NT) {
-      const int ci = R / RH, r = R - ci * RH, i = ci < Q ? ci : ci - Q;
-      const int zs = wrapz(zp - dir_z_rt(i)), ys = wrap_near(y0 - 1 + r - dir_y_rt(i), L.ny);
-      sm.rowp[R] = src + ((long long)ci * L.np + (long long)zs * L.nxny + (long long)ys * L.nx);
+  // Wrapped rows of a y edge, k in [0, YR / 2) of component c: direction i and staged row
+  // r. At the low edge the rows of tile rows -1 (e_y >= 0) and 0 (e_y > 0), whose sources
+  // lie below row 0; at the high edge those of tile rows th and th - 1.
+  __device__ __forceinline__ static void wrapped_row(int k, bool hi_edge, int& i, int& which) {
+    // directions with e_y = +1: 3 7 10 15 17, with e_y = -1: 4 8 9 16 18, e_y = 0 the rest
+    constexpr unsigned long long up = 3ull | 7ull << 5 | 10ull << 10 | 15ull << 15 | 17ull << 20;
+    constexpr unsigned long long dn = 4ull | 8ull << 5 | 9ull << 10 | 16ull << 15 | 18ull << 20;
+    constexpr unsigned long long z0 =
+        0ull | 1ull << 5 | 2ull << 10 | 5ull << 15 | 6ull << 20 | 11ull << 25 | 12ull << 30 | 13ull << 35 | 14ull << 40;
+    if (k < 9) {
+      i = (int)(z0 >> (5 * k)) & 31;
+      which = 0;
+    } else {
+      const int j = k - 9;  // 5 directions, outer row first, then the inner one
+      i = (int)((hi_edge ? dn : up) >> (5 * (j % 5))) & 31;
+      which = j / 5;
     }
   }
-
-  // Copies of the plane whose table is current: this thread's chunk column cj of
-  // rows cr0, cr0 + RS, ...; cx is that column's wrapped x.
-  __device__ __forceinline__ void issue(int cx) {
-    T* to = &sm.stage[0][0][0] + cr0 * SW + cj * E;
-    constexpr int PASSES = (NR + RS - 1) / RS;  // rows cr0 + k RS < NR for every k < PASSES - 1
-    if (cr0 < NR) {
-#pragma unroll
-      for (int k = 0; k < PASSES; ++k) {
-        const int R = cr0 + k * RS;
-        if (k < PASSES - 1 || R < NR) cp_async16(to + k * RS * SW, sm.rowp[R] + cx);
+  __device__ __forceinline__ T* staged_row(int i, int c, int r) { return sm.stage + i * IS + (c * RH + r) * SW; }
+  __device__ __forceinline__ const T* source_row(int i, int c, int r, int zp) const {
+    const int zs = wrapz(zp - dir_z_rt(i)), ys = wrap_near(y0 - 1 + r - dir_y_rt(i), L.ny);
+    return src + ((long long)(c * Q + i) * L.np + (long long)zs * L.nxny + (long long)ys * L.nx);
+  }
+  // This thread's wrapped pieces of plane zp: fetch them into the side buffer, or move
+  // them from there into the staged rows.
+  template <bool FETCH>
+  __device__ __forceinline__ void side_pieces(int zp) {
+    T* side = sm.side;
+    for (int e = left ? 0 : 1; e < (right ? 2 : 1); ++e) {
+      for (int R = threadIdx.x; R < NR; R += NT) {
+        const int i = R / (2 * RH), cr = R - i * 2 * RH, c = cr / RH, r = cr - c * RH;
+        T* piece = side + R * E;
+        if (FETCH) {
+          cp_async16(piece, source_row(i, c, r, zp) + (e == 0 ? L.nx - E : wrap_near(x0 + tw, L.nx)));
+        } else {
+          *reinterpret_cast<int4*>(staged_row(i, c, r) + (e == 0 ? 0 : tw + E)) = *reinterpret_cast<const int4*>(piece);
+        }
       }
+      side += NR * E;
     }
+    for (int e = low ? 0 : 1; e < (high ? 2 : 1); ++e) {
+      for (int q = threadIdx.x; q < YR * CH; q += NT) {
+        const int row = q / CH, j = q - row * CH, c = row >= YR / 2 ? 1 : 0, k = row - c * (YR / 2);
+        int i, which;
+        wrapped_row(k, e == 1, i, which);
+        const int r = e == 0 ? which : th + 1 - which;
+        T* piece = side + q * E;
+        if (FETCH) {
+          cp_async16(piece, source_row(i, c, r, zp) + wrap_near(x0 - E + j * E, L.nx));
+        } else if (r >= 0 && r < RH) {
+          *reinterpret_cast<int4*>(staged_row(i, c, r) + j * E) = *reinterpret_cast<const int4*>(piece);
+        }
+      }
+      if (low && high) side += YR * SW;
+    }
+  }
+
+  // Start the copies of plane p (p in [-1, nz]). Box i is issued by lane i / NW of warp
+  // i % NW, so no warp issues more than a few.
+  __device__ __forceinline__ void issue(int p) {
+    const int zp = wrapz(p);
+    if (threadIdx.x == 0) mbar_expect(&sm.bar, (unsigned)(Q * BOX * (int)sizeof(T)));
+    const int i = (int)(threadIdx.x / 32) + NW * (int)(threadIdx.x % 32);
+    if (i < Q)
+      tma_load5(sm.stage + i * IS, map, x0 - E, y0 - 1 - dir_y_rt(i), wrapz(zp - dir_z_rt(i)), i, 0, &sm.bar);
+    side_pieces<true>(zp);
     cp_async_commit();
+  }
+  // Wait for them; false when they did not land in time.
+  __device__ __forceinline__ bool landed(int p) {
+    const bool ok = mbar_wait(&sm.bar, parity);
+    parity ^= 1u;
+    cp_async_wait_all();
+    side_pieces<false>(wrapz(p));
+    // the next boxes overwrite what these stores wrote
+    asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+    __syncthreads();
+    return ok;
   }
 
   // Population i of component c arriving at tile cell (lx, ly) (ly, lx in [-1, TY] x [-1, TX]):
   // from the staged rows; next to a wall, a population whose source plane is solid
   // is the site's (index s) own opposite one instead.
   template <int I>
-  __device__ __forceinline__ float staged(int c, int ly, int lx) const {
-    return S::cv(sm.stage[c * Q + I][ly + 1][lx + E - dir_x(I)], wgt(I));
+  __device__ __forceinline__ float2 staged(int ly, int lx) const {
+    const T* q = sm.stage + (ly + 1) * SW + lx + E + (I * IS - dir_x(I));
+    return Pair<S>::cv(q[0], q[RH * SW], wgt(I));
   }
   template <int I>
-  __device__ __forceinline__ float pulled(int c, int ly, int lx, bool sol_m, bool sol_p, uint32_t s) const {
+  __device__ __forceinline__ float2 pulled(int ly, int lx, bool sol_m, bool sol_p, uint32_t s) const {
     constexpr int ez = dir_z(I);
-    if (ez != 0 && (ez > 0 ? sol_m : sol_p))
-      return S::ld(src + (long long)(c * Q + opp(I)) * L.np + s, wgt(I));
-    return staged<I>(c, ly, lx);
+    if (ez != 0 && (ez > 0 ? sol_m : sol_p)) {
+      const T* p = src + (long long)opp(I) * L.np + s;
+      return make_float2(S::ld(p, wgt(I)), S::ld(p + (long long)Q * L.np, wgt(I)));
+    }
+    return staged<I>(ly, lx);
   }
 
-  // Read plane p out of the staged rows: the own site into fr/fb, the halo site
+  // Read plane p out of the staged rows: the own site into f, the halo site
   // as sums (the owner's arithmetic, so the halo Psi has the owner's bits); apply the
   // sink and publish Psi to ring slot p & 3. Returns the own site's class.
-  __device__ __forceinline__ int take(int p, bool own, float (&fr)[Q], float (&fb)[Q], float& rr, float& rb) {
+  __device__ __forceinline__ int take(int p, bool own, float2 (&f)[Q], float2& rho) {
     const int zp = wrapz(p), slot = p & 3;
     const bool sol_m = solid_z(L, zp == 0 ? L.nz - 1 : zp - 1), sol_p = solid_z(L, zp == L.nz - 1 ? 0 : zp + 1);
     const int cls = site_class(L, x, y, zp);
-    float pr = 0.0f, pb = 0.0f;
+    float2 ps = make_float2(0.0f, 0.0f);
     const bool walls = sol_m || sol_p;  // the same for the whole plane
     if (cls == SOLID) {
-      rr = rb = 0.0f;
+      rho = ps;
     } else {
       if (!walls) {
         Unroll<0, Q>::run([&](auto ic) {
           constexpr int I = decltype(ic)::value;
-          fr[I] = staged<I>(0, ty, tx);
-          fb[I] = staged<I>(1, ty, tx);
+          f[I] = staged<I>(ty, tx);
         });
       } else {
         const uint32_t s = (uint32_t)(x + L.nx * y) + (uint32_t)L.nxny * (uint32_t)zp;
         Unroll<0, Q>::run([&](auto ic) {
           constexpr int I = decltype(ic)::value;
-          fr[I] = pulled<I>(0, ty, tx, sol_m, sol_p, s);
-          fb[I] = pulled<I>(1, ty, tx, sol_m, sol_p, s);
+          f[I] = pulled<I>(ty, tx, sol_m, sol_p, s);
         });
       }
-      rr = sum19(fr);
-      rb = sum19(fb);
+      rho = sum19(f);
       if (cls == SINK) {
-        if (active && own && own_z(L, zp)) evap += (double)sink_excess(L, fr);
-        sink_densities(L, rr, rb);
+        if (active && own && own_z(L, zp)) evap += (double)sink_excess(L, f);
+        sink_densities(L, rho);
       }
-      pr = psi_of(rr);
-      pb = psi_of(rb);
+      ps = psi_of(rho);
     }
-    sm.ring[slot][ty + 1][tx + 1] = make_float2(pr, pb);
+    sm.ring[slot][ty + 1][tx + 1] = ps;
     if (has_halo) {
       const int hcl = site_class(L, hx, hy, zp);
-      float hpr = 0.0f, hpb = 0.0f;
+      float2 hps = make_float2(0.0f, 0.0f);
       if (hcl != SOLID) {
         // the owner's arithmetic, so the halo Psi has the owner's bits
-        float hrr, hrb;
+        float2 hrho;
         if (!walls) {
-          hrr = sum19_of([&](auto ic) { return staged<decltype(ic)::value>(0, hly, hlx); });
-          hrb = sum19_of([&](auto ic) { return staged<decltype(ic)::value>(1, hly, hlx); });
+          hrho = sum19_of<float2>([&](auto ic) { return staged<decltype(ic)::value>(hly, hlx); });
         } else {
           const uint32_t s = (uint32_t)(hx + L.nx * hy) + (uint32_t)L.nxny * (uint32_t)zp;
-          hrr = sum19_of([&](auto ic) { return pulled<decltype(ic)::value>(0, hly, hlx, sol_m, sol_p, s); });
-          hrb = sum19_of([&](auto ic) { return pulled<decltype(ic)::value>(1, hly, hlx, sol_m, sol_p, s); });
+          hrho = sum19_of<float2>([&](auto ic) { return pulled<decltype(ic)::value>(hly, hlx, sol_m, sol_p, s); });
         }
-        if (hcl == SINK) sink_densities(L, hrr, hrb);
-        hpr = psi_of(hrr);
-        hpb = psi_of(hrb);
+        if (hcl == SINK) sink_densities(L, hrho);
+        hps = psi_of(hrho);
       }
-      sm.ring[slot][hly + 1][hlx + 1] = make_float2(hpr, hpb);
+      sm.ring[slot][hly + 1][hlx + 1] = hps;
     }
     return cls;
   }
 
   // Collide plane z (in [0, nz); read out one plane earlier) and store f*.
-  __device__ __forceinline__ void finish(int z, float (&fr)[Q], float (&fb)[Q], float rr, float rb, int cls) {
+  __device__ __forceinline__ void finish(int z, float2 (&f)[Q], float2 rho, int cls) {
     if (!active || cls == SOLID) return;
     const int s = x + L.nx * y + L.nxny * z;
     if (cls == SINK) {
 #pragma unroll
-      for (int i = 0; i < Q; ++i) { fr[i] = rest_pop(i, rr); fb[i] = rest_pop(i, rb); }
+      for (int i = 0; i < Q; ++i) f[i] = rest_pop(i, rho);
     } else {
-      float ar[3], ab[3];
-      auto psi2 = [&](int sl, int ly, int lx) { return sm.ring[sl][ly + 1][lx + 1]; };
-      force_sums(psi2, (z - 1) & 3, z & 3, (z + 1) & 3, ty, tx, ar, ab);
-      const float2 ps = sm.ring[z & 3][ty + 1][tx + 1];
-      collide(L, fr, fb, rr, rb, ps.x, ps.y, ar, ab);
+      float2 a[3];
+      auto psi = [&](int sl, int ly, int lx) { return sm.ring[sl][ly + 1][lx + 1]; };
+      force_sums(psi, (z - 1) & 3, z & 3, (z + 1) & 3, ty, tx, a);
+      collide(L, f, rho, sm.ring[z & 3][ty + 1][tx + 1], a);
     }
-    store_site<S>(L, dst, s, fr, fb);
+    store_site<S>(L, dst, s, f);
   }
 
-  __device__ __forceinline__ void run(int zb, int ze, bool down) {
-    float cr[Q], cb[Q], nr[Q], nb[Q];
-    float crr = 0.f, crb = 0.f, nrr = 0.f, nrb = 0.f;
+  // Returns false when a plane's copies did not land in time (the CTA stops marching).
+  __device__ __forceinline__ bool run(int zb, int ze, bool down) {
+    float2 c[Q], n2[Q];
+    float2 crho = make_float2(0.f, 0.f), nrho = crho;
     int ccl = SOLID;
     const int d = down ? -1 : 1;
     const int first = down ? ze - 1 : zb;
     const int n = ze - zb;
-    table(first - d);
-    __syncthreads();  // chunk and row tables
-    const int cx = sm.chx[cj];
-    issue(cx);
+    issue(first - d);
     for (int o = 0; o < n + 2; ++o) {
       const int p = first + (o - 1) * d;
-      cp_async_wait_all();
-      __syncthreads();  // every thread's copies of plane p have landed
-      const int pcl = take(p, o >= 1 && o <= n, nr, nb, nrr, nrb);
-      if (o + 1 < n + 2) table(p + d);
-      __syncthreads();  // ring complete, staged rows read out, next table written
-      if (o + 1 < n + 2) issue(cx);
-      if (o >= 2) finish(p - d, cr, cb, crr, crb, ccl);
+      const bool ok = landed(p);
+      const int pcl = take(p, o >= 1 && o <= n, n2, nrho);
+      // ring complete, staged rows read out
+      if (__syncthreads_or(!ok)) {
+        if (!ok) mbar_wait(&sm.bar, parity ^ 1u);  // no copy may land after the CTA has gone
+        return false;
+      }
+      if (o + 1 < n + 2) issue(p + d);
+      if (o >= 2) finish(p - d, c, crho, ccl);
 #pragma unroll
-      for (int i = 0; i < Q; ++i) { cr[i] = nr[i]; cb[i] = nb[i]; }
-      crr = nrr;
-      crb = nrb;
+      for (int i = 0; i < Q; ++i) c[i] = n2[i];
+      crho = nrho;
       ccl = pcl;
     }
+    return true;
   }
 
   __device__ __forceinline__ double block_evap() {
@@ -955,47 +1113,44 @@ __device__ __forceinline__ void aa_slot(const PullIdx& P, int& idx, int& d) {
 
 // Arrived populations of the site of P (plain loads: the lattice is written in place).
 template <class S, bool ODD>
-__device__ __forceinline__ void aa_load(const LatDev& L, const typename S::T* A, const PullIdx& P, float (&fr)[Q],
-                                        float (&fb)[Q]) {
+__device__ __forceinline__ void aa_load(const LatDev& L, const typename S::T* A, const PullIdx& P,
+                                        float2 (&f)[Q]) {
   const long long cstride = (long long)Q * L.np;
   Unroll<0, Q>::run([&](auto ic) {
     constexpr int I = decltype(ic)::value;
     int idx, d;
     aa_slot<I, ODD>(P, idx, d);
     const typename S::T* p = A + (long long)d * L.np + idx;
-    fr[I] = S::cv(p[0], wgt(I));
-    fb[I] = S::cv(p[cstride], wgt(I));
+    f[I] = Pair<S>::cv(p[0], p[cstride], wgt(I));
   });
 }
 
 // The same loads at L2 only (the persistent in-place step, where neighbouring CTAs
 // rewrite slots this CTA read in an earlier step).
 template <class S, bool ODD>
-__device__ __forceinline__ void aa_load_cg(const LatDev& L, const typename S::T* A, const PullIdx& P, float (&fr)[Q],
-                                           float (&fb)[Q]) {
+__device__ __forceinline__ void aa_load_cg(const LatDev& L, const typename S::T* A, const PullIdx& P,
+                                           float2 (&f)[Q]) {
   const long long cstride = (long long)Q * L.np;
   Unroll<0, Q>::run([&](auto ic) {
     constexpr int I = decltype(ic)::value;
     int idx, d;
     aa_slot<I, ODD>(P, idx, d);
     const typename S::T* p = A + (long long)d * L.np + idx;
-    fr[I] = S::ldcg(p, wgt(I));
-    fb[I] = S::ldcg(p + cstride, wgt(I));
+    f[I] = make_float2(S::ldcg(p, wgt(I)), S::ldcg(p + cstride, wgt(I)));
   });
 }
 
 // f*_j into the slot population opp(j) was read from.
 template <class S, bool ODD>
-__device__ __forceinline__ void aa_store(const LatDev& L, typename S::T* A, const PullIdx& P, const float (&fr)[Q],
-                                         const float (&fb)[Q]) {
+__device__ __forceinline__ void aa_store(const LatDev& L, typename S::T* A, const PullIdx& P,
+                                         const float2 (&f)[Q]) {
   const long long cstride = (long long)Q * L.np;
   Unroll<0, Q>::run([&](auto jc) {
     constexpr int J = decltype(jc)::value;
     int idx, d;
     aa_slot<opp(J), ODD>(P, idx, d);
     typename S::T* p = A + (long long)d * L.np + idx;
-    S::st(p, fr[J], wgt(J));
-    S::st(p + cstride, fb[J], wgt(J));
+    Pair<S>::st(p, p + cstride, f[J], wgt(J));
   });
 }
 

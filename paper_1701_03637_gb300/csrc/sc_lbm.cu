@@ -60,29 +60,42 @@ int wrap_host(int v, int n) { return ((v % n) + n) % n; }
 // ------------------------------------------------------------------ kernels
 
 // Persistent fused step; Rows selects the staged-rows marcher (TileRows) over
-// the per-thread one (Tile). CTA b marches items [starts[b], starts[b + 1]) of
-// the host-built work list (see plan_launch): tile columns of TX x TY sites and
-// z chunks, in every round the resident CTAs on neighbouring columns of the
-// same chunk in lock-step, so that a column's halo and shifted-pull sectors are
-// read from DRAM once and then from L2 by its neighbours.
+// the per-thread one (Tile). The host-built work list (plan_launch) holds tile columns of
+// TX x TY sites and z chunks, chunk-major; CTAs claim its items in order from a counter,
+// so that at any time the CTAs work on neighbouring columns of the same chunk, a fraction
+// of a plane apart, and a column's halo and shifted-pull sectors are read from DRAM once
+// and then from L2 by its neighbours, whatever each CTA's speed. (Dealt out round-robin,
+// slower CTAs fell further behind with every item.) CTA b's first
+// item is item b. The counter wraps to 0 with the last claim of the launch (items past the
+// first per CTA, and one failing claim per CTA).
 template <int TX, int TY, class S, bool Rows>
 __global__ void __launch_bounds__(TX * TY, (512 / (TX * TY)) > 1 ? 512 / (TX * TY) : 1)
     k_step(const LatDev L, const typename S::T* __restrict__ src, typename S::T* __restrict__ dst,
-           double* __restrict__ evap_cum, int cols_x, const int4* __restrict__ items, const int* __restrict__ starts) {
+           double* __restrict__ evap_cum, int nslots, int cols_x, const int4* __restrict__ items, int nitems,
+           unsigned* __restrict__ next, const __grid_constant__ CUtensorMap map, int* __restrict__ err) {
   using TileT = std::conditional_t<Rows, TileRows<TX, TY, S>, Tile<TX, TY, S>>;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
+  extern __shared__ __align__(128) unsigned char smem_raw[];
   auto& sm = *reinterpret_cast<typename TileT::Smem*>(smem_raw);
-  TileT t(L, sm, src, dst);
-  const int i0 = starts[blockIdx.x], i1 = starts[blockIdx.x + 1];
-  for (int it = i0; it < i1; ++it) {
-    const int4 w = items[it];  // tile column, first plane, end plane, downward
-    if (it > i0) __syncthreads();  // the previous item's last reads of the ring
-    t.setup(w.x % cols_x, w.x / cols_x);
-    t.run(w.y, w.z, w.w != 0);
-  }
-  if (L.geometry != 0) {
-    const double e = t.block_evap();
-    if (threadIdx.x == 0) evap_cum[blockIdx.x] += e;
+  __shared__ int s_it[2];
+  TileT t(L, sm, src, dst, &map);
+  const int G = (int)gridDim.x;  // at most nitems
+  int turn = 0;
+  bool ok = true;
+  for (int it = (int)blockIdx.x; it < nitems; it = s_it[turn ^= 1]) {
+    if (threadIdx.x == 0) s_it[turn ^ 1] = G + (int)atomicInc(next, (unsigned)nitems - 1u);  // one item ahead
+    if (ok) {
+      const int4 w = items[it];  // tile column, first plane, end plane, downward
+      t.setup(w.x % cols_x, w.x / cols_x);
+      ok = t.run(w.y, w.z, w.w != 0);
+      if (!ok && threadIdx.x == 0) *err = 3;
+    }
+    if (L.geometry != 0 && __syncthreads_or(t.evap != 0.0)) {
+      const double e = t.block_evap();
+      // a slot per item; launches with more items than slots share them
+      if (threadIdx.x == 0) atomicAdd(evap_cum + it % nslots, e);
+      t.evap = 0.0;
+    }
+    __syncthreads();  // the item's last reads of the ring, and the next item's number
   }
 }
 
@@ -118,11 +131,11 @@ __global__ void __launch_bounds__(kAAThreads) k_aa_psi(const LatDev L, const typ
     const PullIdx P(L, r.x, r.y, r.z);
     float2 v = make_float2(0.f, 0.f);
     if (cls != SOLID) {
-      float fr[Q], fb[Q];
-      aa_load<S, ODD>(L, A, P, fr, fb);
-      float rr = sum19(fr), rb = sum19(fb);
-      if (cls == SINK) sink_densities(L, rr, rb);
-      v = make_float2(psi_of(rr), psi_of(rb));
+      float2 f[Q];
+      aa_load<S, ODD>(L, A, P, f);
+      float2 rho = sum19(f);
+      if (cls == SINK) sink_densities(L, rho);
+      v = psi_of(rho);
     }
     psi[P.s] = v;
   }
@@ -142,15 +155,15 @@ __global__ void __launch_bounds__(kAAThreads, 4) k_aa_collide(const LatDev L, ty
     const int cls = site_class(L, r.x, r.y, r.z);
     if (cls == SOLID) continue;
     const PullIdx P(L, r.x, r.y, r.z);
-    float fr[Q], fb[Q];
-    aa_load<S, ODD>(L, A, P, fr, fb);
-    float rr = sum19(fr), rb = sum19(fb);
+    float2 f[Q];
+    aa_load<S, ODD>(L, A, P, f);
+    float2 rho = sum19(f);
     if (cls == SINK) {
       // neither forced nor collided: f^eq at rest of the reset densities
-      evap += (double)sink_excess(L, fr);
-      sink_densities(L, rr, rb);
+      evap += (double)sink_excess(L, f);
+      sink_densities(L, rho);
 #pragma unroll
-      for (int i = 0; i < Q; ++i) { fr[i] = rest_pop(i, rr); fb[i] = rest_pop(i, rb); }
+      for (int i = 0; i < Q; ++i) f[i] = rest_pop(i, rho);
     } else {
       const int nx = L.nx, ny = L.ny;
       auto psi2 = [&](int zb, int yy, int xx) {
@@ -158,12 +171,11 @@ __global__ void __launch_bounds__(kAAThreads, 4) k_aa_collide(const LatDev L, ty
         xx = xx < 0 ? xx + nx : (xx >= nx ? xx - nx : xx);
         return psi[zb + yy * nx + xx];
       };
-      float ar[3], ab[3];
-      force_sums(psi2, P.zs[2], P.zs[1], P.zs[0], r.y, r.x, ar, ab);  // planes z - 1, z, z + 1
-      const float2 ps = psi[P.s];
-      collide(L, fr, fb, rr, rb, ps.x, ps.y, ar, ab);
+      float2 a[3];
+      force_sums(psi2, P.zs[2], P.zs[1], P.zs[0], r.y, r.x, a);  // planes z - 1, z, z + 1
+      collide(L, f, rho, psi[P.s], a);
     }
-    aa_store<S, ODD>(L, A, P, fr, fb);
+    aa_store<S, ODD>(L, A, P, f);
   }
   if (L.geometry != 0) {
     __shared__ double red[kAAThreads / 32];
@@ -241,12 +253,6 @@ __device__ __forceinline__ unsigned long long ld_acquire_u64(const unsigned long
 __device__ __forceinline__ void st_release_u64(unsigned long long* p, unsigned long long v) {
   asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
-__device__ __forceinline__ unsigned long long global_ns() {
-  unsigned long long t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-  return t;
-}
-
 // Polled by threads 0..8 before a barrier: whether tile column (bx + dx, by + dy)
 // (periodic; dx, dy in {-1, 0, 1} from the thread index, the CTA itself included)
 // has counter >= target. False when the wait gave up (time limit, or another CTA
@@ -306,11 +312,11 @@ struct PersistTile {
         } else if (hx == tw && right_saved) {
           v = __ldcg(edge_at(a.B - 1, zq, y));
         } else {
-          float fr[Q], fb[Q];
-          aa_load_cg<S, ODD>(L, A, PullIdx(L, x, y, zq), fr, fb);
-          float rr = sum19(fr), rb = sum19(fb);
-          if (site_class(L, x, y, zq) == SINK) sink_densities(L, rr, rb);
-          v = make_float2(psi_of(rr), psi_of(rb));
+          float2 f[Q];
+          aa_load_cg<S, ODD>(L, A, PullIdx(L, x, y, zq), f);
+          float2 rho = sum19(f);
+          if (site_class(L, x, y, zq) == SINK) sink_densities(L, rho);
+          v = psi_of(rho);
         }
       }
       cell(sa, c) = v;
@@ -333,22 +339,21 @@ struct PersistTile {
       const int cls = site_class(L, x, y, p);
       if (cls == SOLID) continue;
       const PullIdx P(L, x, y, p);
-      float fr[Q], fb[Q];
-      aa_load_cg<S, ODD>(L, A, P, fr, fb);
-      float rr = sum19(fr), rb = sum19(fb);
+      float2 f[Q];
+      aa_load_cg<S, ODD>(L, A, P, f);
+      float2 rho = sum19(f);
       if (cls == SINK) {
-        evap += (double)sink_excess(L, fr);
-        sink_densities(L, rr, rb);
+        evap += (double)sink_excess(L, f);
+        sink_densities(L, rho);
 #pragma unroll
-        for (int i = 0; i < Q; ++i) { fr[i] = rest_pop(i, rr); fb[i] = rest_pop(i, rb); }
+        for (int i = 0; i < Q; ++i) f[i] = rest_pop(i, rho);
       } else {
         auto psi2 = [&](int sl, int yy, int xx) { return cell(sl, (yy + 1) * RW + (xx + 1)); };
-        float ar[3], ab[3];
-        force_sums(psi2, sm1, s0, sp1, ly, lx, ar, ab);
-        const float2 ps = cell(s0, (ly + 1) * RW + (lx + 1));
-        collide(L, fr, fb, rr, rb, ps.x, ps.y, ar, ab);
+        float2 fa[3];
+        force_sums(psi2, sm1, s0, sp1, ly, lx, fa);
+        collide(L, f, rho, cell(s0, (ly + 1) * RW + (lx + 1)), fa);
       }
-      aa_store<S, ODD>(L, A, P, fr, fb);
+      aa_store<S, ODD>(L, A, P, f);
     }
   }
 
@@ -430,9 +435,9 @@ __global__ void __launch_bounds__(NT, 512 / NT)
 // buffer or of the in-place lattice's even form, or the odd form's own slots.
 template <class S>
 __device__ __forceinline__ void arrived(const LatDev& L, const typename S::T* __restrict__ src, const PullIdx& P,
-                                        int odd, float (&fr)[Q], float (&fb)[Q]) {
-  if (odd) aa_load<S, true>(L, src, P, fr, fb);
-  else pull_full<S>(L, src, P, fr, fb);
+                                        int odd, float2 (&f)[Q]) {
+  if (odd) aa_load<S, true>(L, src, P, f);
+  else pull_full<S>(L, src, P, f);
 }
 
 __device__ __forceinline__ void site_of(const LatDev& L, long long s, int& x, int& y, int& z) {
@@ -452,28 +457,27 @@ __global__ void k_canonical(const LatDev L, const typename S::T* __restrict__ sr
     int x, y, z;
     site_of(L, s, x, y, z);
     const int cls = site_class(L, x, y, z);
-    float fr[Q], fb[Q], rr = 0.f, rb = 0.f;
+    float2 f[Q], rho = make_float2(0.f, 0.f);
     if (cls == SOLID) {
 #pragma unroll
-      for (int i = 0; i < Q; ++i) fr[i] = fb[i] = 0.f;
+      for (int i = 0; i < Q; ++i) f[i] = rho;
     } else {
       const PullIdx P(L, x, y, z);
-      arrived<S>(L, src, P, odd, fr, fb);
-      rr = sum19(fr);
-      rb = sum19(fb);
+      arrived<S>(L, src, P, odd, f);
+      rho = sum19(f);
       if (cls == SINK) {
-        sink_densities(L, rr, rb);
+        sink_densities(L, rho);
 #pragma unroll
-        for (int i = 0; i < Q; ++i) { fr[i] = rest_pop(i, rr); fb[i] = rest_pop(i, rb); }
+        for (int i = 0; i < Q; ++i) f[i] = rest_pop(i, rho);
       }
     }
     const long long o = s - s0;
-    if (rho_out) { rho_out[o] = rr; rho_out[rho_stride + o] = rb; }
+    if (rho_out) { rho_out[o] = rho.x; rho_out[rho_stride + o] = rho.y; }
     if (f_out) {
 #pragma unroll
       for (int i = 0; i < Q; ++i) {
-        f_out[(long long)i * f_stride + o] = fr[i];
-        f_out[(long long)(Q + i) * f_stride + o] = fb[i];
+        f_out[(long long)i * f_stride + o] = f[i].x;
+        f_out[(long long)(Q + i) * f_stride + o] = f[i].y;
       }
     }
   }
@@ -500,21 +504,21 @@ __global__ void __launch_bounds__(kDiagThreads) k_diag(const LatDev L, const typ
       const int x = q % L.nx, y = q / L.nx;
       const int cls = site_class(L, x, y, z);
       const PullIdx P(L, x, y, z);
-      float fr[Q], fb[Q];
-      arrived<S>(L, src, P, odd, fr, fb);
-      float rr = sum19(fr), rb = sum19(fb);
-      double mr = rr;
+      float2 f[Q];
+      arrived<S>(L, src, P, odd, f);
+      float2 rho = sum19(f);
+      double mr = rho.x;
       if (cls == SINK) {
-        acc[3] += (double)sink_excess(L, fr);
-        sink_densities(L, rr, rb);
+        acc[3] += (double)sink_excess(L, f);
+        sink_densities(L, rho);
         mr = L.rhoH_mass;
-        if (rb < 0.0f) acc[6] = 1.0;
+        if (rho.y < 0.0f) acc[6] = 1.0;
       }
-      if (!isfinite(rr) || !isfinite(rb)) acc[5] = 1.0;
+      if (!isfinite(rho.x) || !isfinite(rho.y)) acc[5] = 1.0;
       acc[0] += mr;
-      acc[1] += rb;
-      acc[2] += (double)rr - (double)rb;
-      acc[4] += rr > rb ? 1.0 : 0.0;
+      acc[1] += rho.y;
+      acc[2] += (double)rho.x - (double)rho.y;
+      acc[4] += rho.x > rho.y ? 1.0 : 0.0;
     }
   }
   __shared__ double red[kDiagThreads / 32][NF];
@@ -548,20 +552,20 @@ __global__ void __launch_bounds__(kDiagThreads) k_diag(const LatDev L, const typ
 // FP64 densities of the canonical populations of site (x, y, z); returns its class.
 template <class S>
 __device__ __forceinline__ int canonical_rho(const LatDev& L, const typename S::T* __restrict__ src, int odd, int x,
-                                             int y, int z, double& rr, double& rb, float (&fr)[Q], float (&fb)[Q]) {
+                                             int y, int z, double& rr, double& rb, float2 (&f)[Q]) {
   const int cls = site_class(L, x, y, z);
   rr = rb = 0.0;
   if (cls == SOLID) return cls;
   const PullIdx P(L, x, y, z);
-  arrived<S>(L, src, P, odd, fr, fb);
+  arrived<S>(L, src, P, odd, f);
   if (cls == SINK) {
-    float a = sum19(fr), b = sum19(fb);
-    sink_densities(L, a, b);
+    float2 rho = sum19(f);
+    sink_densities(L, rho);
 #pragma unroll
-    for (int i = 0; i < Q; ++i) { fr[i] = rest_pop(i, a); fb[i] = rest_pop(i, b); }
+    for (int i = 0; i < Q; ++i) f[i] = rest_pop(i, rho);
   }
 #pragma unroll
-  for (int i = 0; i < Q; ++i) { rr += (double)fr[i]; rb += (double)fb[i]; }
+  for (int i = 0; i < Q; ++i) { rr += (double)f[i].x; rb += (double)f[i].y; }
   return cls;
 }
 
@@ -576,24 +580,24 @@ __global__ void __launch_bounds__(kDiagThreads) k_flux(const LatDev L, const typ
   double acc[3] = {0.0, 0.0, 0.0};
   for (int q = b + threadIdx.x; q < e; q += blockDim.x) {
     const int x = q % L.nx, y = q / L.nx;
-    float fr[Q], fb[Q];
+    float2 f[Q];
     double rr, rb;
-    if (canonical_rho<S>(L, src, odd, x, y, z, rr, rb, fr, fb) != FLUID) continue;
+    if (canonical_rho<S>(L, src, odd, x, y, z, rr, rb, f) != FLUID) continue;
     double mr[3] = {0.0, 0.0, 0.0}, mb[3] = {0.0, 0.0, 0.0}, ar[3] = {0.0, 0.0, 0.0}, ab[3] = {0.0, 0.0, 0.0};
 #pragma unroll
     for (int i = 1; i < Q; ++i) {
       const double e[3] = {(double)dir_x(i), (double)dir_y(i), (double)dir_z(i)};
 #pragma unroll
-      for (int d = 0; d < 3; ++d) { mr[d] += e[d] * (double)fr[i]; mb[d] += e[d] * (double)fb[i]; }
+      for (int d = 0; d < 3; ++d) { mr[d] += e[d] * (double)f[i].x; mb[d] += e[d] * (double)f[i].y; }
     }
     // sum_i w_i Psi(x + e_i) e_i of both components over the 18 neighbours
 #pragma unroll 1
     for (int i = 1; i < Q; ++i) {
       const int ex = dir_x(i), ey = dir_y(i), ez = dir_z(i);
-      float gr[Q], gb[Q];
+      float2 fn[Q];
       double nr, nb;
       const int cls = canonical_rho<S>(L, src, odd, wrap_near(x + ex, L.nx), wrap_near(y + ey, L.ny),
-                                       wrap_near(z + ez, L.nz), nr, nb, gr, gb);
+                                       wrap_near(z + ez, L.nz), nr, nb, fn);
       const double pr = cls == SOLID ? 0.0 : 1.0 - exp(-nr), pb = cls == SOLID ? 0.0 : 1.0 - exp(-nb);
       const double w = wgt_d(i);
       ar[0] += w * pr * ex; ar[1] += w * pr * ey; ar[2] += w * pr * ez;
@@ -711,17 +715,15 @@ __global__ void k_load(const LatDev L, typename S::T* __restrict__ dst, long lon
     const int cls = site_class(L, x, y, z);
     if (cls == SOLID) continue;
     const long long o = s - s0;
-    float fr[Q], fb[Q];
+    float2 f[Q];
     if (mode == 0) {
 #pragma unroll
-      for (int i = 0; i < Q; ++i) {
-        fr[i] = f_in[(long long)i * f_stride + o];
-        fb[i] = f_in[(long long)(Q + i) * f_stride + o];
-      }
+      for (int i = 0; i < Q; ++i)
+        f[i] = make_float2(f_in[(long long)i * f_stride + o], f_in[(long long)(Q + i) * f_stride + o]);
     } else if (mode == 1) {
-      const float r = rho_in[o], b = rho_in[rho_stride + o];
+      const float2 rho = make_float2(rho_in[o], rho_in[rho_stride + o]);
 #pragma unroll
-      for (int i = 0; i < Q; ++i) { fr[i] = wgt(i) * r; fb[i] = wgt(i) * b; }
+      for (int i = 0; i < Q; ++i) f[i] = rest_pop(i, rho);
     } else {
       bool rich;
       const int zg = global_z(L, z);  // the shape and the noise are the whole lattice's
@@ -738,16 +740,13 @@ __global__ void k_load(const LatDev L, typename S::T* __restrict__ dst, long lon
       const double r = (rich ? sh.hi : sh.lo) + __dmul_rn(sh.amp, __dadd_rn(2.0 * ur, -1.0));
       const double b = (rich ? sh.lo : sh.hi) + __dmul_rn(sh.amp, __dadd_rn(2.0 * ub, -1.0));
 #pragma unroll
-      for (int i = 0; i < Q; ++i) {
-        fr[i] = (float)__dmul_rn(wgt_d(i), r);
-        fb[i] = (float)__dmul_rn(wgt_d(i), b);
-      }
+      for (int i = 0; i < Q; ++i) f[i] = make_float2((float)__dmul_rn(wgt_d(i), r), (float)__dmul_rn(wgt_d(i), b));
     }
     if (cls == SINK) {
-      float rr = sum19(fr), rb = sum19(fb);
-      sink_densities(L, rr, rb);
+      float2 rho = sum19(f);
+      sink_densities(L, rho);
 #pragma unroll
-      for (int i = 0; i < Q; ++i) { fr[i] = rest_pop(i, rr); fb[i] = rest_pop(i, rb); }
+      for (int i = 0; i < Q; ++i) f[i] = rest_pop(i, rho);
     }
     // inverse of the pull: f_i(x) is read from x - e_i (wrapped), or from (x, opp(i))
     // when plane z - e_iz is solid.
@@ -760,8 +759,7 @@ __global__ void k_load(const LatDev L, typename S::T* __restrict__ dst, long lon
                           : wrapi(x - dir_x(I), L.nx) + L.nx * wrapi(y - dir_y(I), L.ny) + L.nxny * zs;
       const int d = sol ? opp(I) : I;
       typename S::T* p = dst + (long long)d * L.np + idx;
-      S::st(p, fr[I], wgt(I));
-      S::st(p + cstride, fb[I], wgt(I));
+      Pair<S>::st(p, p + cstride, f[I], wgt(I));
     });
   }
 }
@@ -773,22 +771,30 @@ struct StepArgs {
   const void* src;
   void* dst;
   double* evap;
+  int nslots;  // evaporated-mass slots
   int cols_x;
   const int4* items;
-  const int* starts;
+  int nitems;
+  unsigned* next;  // claim counter, 0 between launches
   int G;
   cudaStream_t st;
+  CUtensorMap map;  // of src, with the tile's box (staged rows)
+  int* err;         // set to 3 when a plane's copies do not land in time
 };
 
+// Dynamic shared memory; staged rows need a side buffer per lattice edge that one tile
+// touches (two in x or y where a tile spans the lattice).
 template <int TX, int TY, class S, bool Rows = false>
-constexpr size_t step_smem() {
-  return Rows ? sizeof(typename TileRows<TX, TY, S>::Smem) : sizeof(typename Tile<TX, TY, S>::Smem);
+constexpr size_t step_smem(const LatDev& L) {
+  return Rows ? TileRows<TX, TY, S>::smem_bytes(L.nx <= TX ? 2 : 1, L.ny < TY + 2 ? 2 : 1)
+              : sizeof(typename Tile<TX, TY, S>::Smem);
 }
 
 template <int TX, int TY, class S, bool Rows>
 cudaError_t launch_step(const StepArgs& a) {
-  k_step<TX, TY, S, Rows><<<a.G, TX * TY, step_smem<TX, TY, S, Rows>(), a.st>>>(
-      a.L, (const typename S::T*)a.src, (typename S::T*)a.dst, a.evap, a.cols_x, a.items, a.starts);
+  k_step<TX, TY, S, Rows><<<a.G, TX * TY, step_smem<TX, TY, S, Rows>(a.L), a.st>>>(
+      a.L, (const typename S::T*)a.src, (typename S::T*)a.dst, a.evap, a.nslots, a.cols_x, a.items, a.nitems, a.next, a.map,
+      a.err);
   return cudaGetLastError();
 }
 
@@ -796,13 +802,14 @@ cudaError_t launch_step(const StepArgs& a) {
 // dynamic shared memory there (above the 48 KB default); every handle calls this
 // on its device before its first step.
 template <int TX, int TY, class S, bool Rows>
-int occupancy_step() {
+int occupancy_step(const LatDev& L) {
   int nb = 0;
-  if (cudaFuncSetAttribute(k_step<TX, TY, S, Rows>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)step_smem<TX, TY, S, Rows>()) != cudaSuccess)
+  const size_t smem = step_smem<TX, TY, S, Rows>(L);
+  // the attribute is the kernel's, not the handle's: its largest use
+  constexpr size_t most = Rows ? TileRows<TX, TY, S>::smem_bytes(2, 2) : sizeof(typename Tile<TX, TY, S>::Smem);
+  if (cudaFuncSetAttribute(k_step<TX, TY, S, Rows>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most) != cudaSuccess)
     return 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_step<TX, TY, S, Rows>, TX * TY,
-                                                    step_smem<TX, TY, S, Rows>()) != cudaSuccess)
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_step<TX, TY, S, Rows>, TX * TY, smem) != cudaSuccess)
     return 0;
   return nb;
 }
@@ -810,7 +817,7 @@ int occupancy_step() {
 using LaunchFn = cudaError_t (*)(const StepArgs&);
 struct StepOps {
   LaunchFn launch;
-  int (*occupancy)();  // resident CTAs per SM
+  int (*occupancy)(const LatDev&);  // resident CTAs per SM
 };
 
 template <class S, bool Rows>
@@ -849,7 +856,7 @@ struct Layout {
   long long units, nslots;
   int diag_nsplit;
   long long cap_items;         // work-list capacity (items of any tile shape and schedule)
-  size_t off_pop[2], off_psi, off_stage, off_evap, off_diag, off_items, off_starts, off_flags, total;
+  size_t off_pop[2], off_psi, off_stage, off_evap, off_diag, off_items, off_flags, total;
 };
 
 int auto_tile(const sc_params* p) {
@@ -892,12 +899,12 @@ Layout make_layout(const sc_params* p) {
   l.off_stage = off; off += align256((size_t)2 * l.stage_n * sizeof(float));
   l.off_evap = off; off += align256((size_t)l.nslots * sizeof(double));
   l.off_diag = off; off += align256((size_t)p->nz * l.diag_nsplit * kDiagFields * sizeof(double));
-  // work list: at most one item per (column of the smallest tile, plane), plus one
-  // split per CTA of the balanced schedule (under 1 byte per site)
-  l.cap_items = (long long)((p->nx + 7) / 8) * ((p->ny + 3) / 4) * p->nz + kMaxCtas;
+  // work list: at most one item per (column of the smallest tile, plane) (under 1 byte
+  // per site)
+  l.cap_items = (long long)((p->nx + 7) / 8) * ((p->ny + 3) / 4) * p->nz;
   l.off_items = off; off += align256((size_t)l.cap_items * sizeof(int4));
-  l.off_starts = off; off += align256((size_t)(kMaxCtas + 1) * sizeof(int));
-  // progress counters of the persistent in-place step (two per CTA) and its error word
+  // progress counters of the persistent in-place step (two per CTA), its error word, and
+  // the claim counter of the two-lattice step
   l.off_flags = off; off += align256((size_t)2 * kMaxCtas * sizeof(unsigned long long) + 256);
   l.total = off;
   return l;
@@ -970,6 +977,8 @@ struct sc_lbm {
   double evap_offset;  // evaporated mass restored by sc_lbm_set_counters
   double* h_diag;      // pinned
   double* h_evap;      // pinned
+  int* h_err;          // pinned, written by a step whose copies did not land in time
+  CUtensorMap maps[2]; // of the two population buffers, with the tile's box (staged rows)
   int grid;  // CTAs of the persistent step (in place: of k_aa_collide)
   int grid_psi;  // CTAs of k_aa_psi
   // persistent in-place step (k_aa_persist), when the layout is in place and it fits
@@ -985,6 +994,7 @@ struct sc_lbm {
   const char* persist_why;   // why the persistent step was not planned
   bool slab;                 // z-slab of a larger lattice (sc_slab_create)
   int zmax;  // planes of the longest work item
+  int nitems;  // work items of a step (two lattices)
   cudaGraphExec_t graph;
   int graph_len;
   int graph_cur;
@@ -996,34 +1006,63 @@ struct sc_lbm {
   double* evap() const { return (double*)(base + lay.off_evap); }
   double* diag() const { return (double*)(base + lay.off_diag); }
   int4* items() const { return (int4*)(base + lay.off_items); }
-  int* starts() const { return (int*)(base + lay.off_starts); }
   unsigned long long* flags() const { return (unsigned long long*)(base + lay.off_flags); }
+  unsigned* next() const { return (unsigned*)(err() + 16); }
   int* err() const { return (int*)(base + lay.off_flags + 2 * kMaxCtas * sizeof(unsigned long long)); }
 };
 
 namespace {
 
 // Launch configuration of the persistent step for one tile shape: the grid and
-// the work list, CTA b taking items [starts[b], starts[b + 1]).
+// the work list, whose items the CTAs claim in order.
 struct LaunchCfg {
   int tile, cols_x, cols, grid, zmax;
   std::vector<int4> items;  // tile column, first plane, end plane, downward
-  std::vector<int> starts;
 };
+
+// Tensor map of a population buffer for the staged rows of a tile shape: dimensions
+// (x, y, z, direction, component), a box of one direction's TX + 2 E columns and TY + 2
+// rows of one plane, both components.
+using EncodeFn = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
+                              const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
+                              CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+int encode_map(const sc_lbm* h, const void* pop, int tile, CUtensorMap* m) {
+  static EncodeFn encode = nullptr;
+  static std::once_flag once;
+  std::call_once(once, [] {
+    void* fn = nullptr;
+    cudaDriverEntryPointQueryResult q{};
+    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &q) == cudaSuccess &&
+        q == cudaDriverEntryPointSuccess)
+      encode = (EncodeFn)fn;
+  });
+  if (!encode) return fail(SC_ECUDA, "the driver has no cuTensorMapEncodeTiled");
+  const cuuint64_t es = elem_size(h->p.storage);
+  const CUtensorMapDataType type = h->p.storage == SC_STORAGE_F32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32
+                                 : h->p.storage == SC_STORAGE_BF16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16
+                                                                   : CU_TENSOR_MAP_DATA_TYPE_FLOAT16;
+  const cuuint64_t nx = h->p.nx, ny = h->p.ny, np = h->lay.np;
+  const cuuint64_t dims[5] = {nx, ny, (cuuint64_t)h->p.nz, Q, 2};
+  const cuuint64_t strides[4] = {nx * es, nx * ny * es, np * es, Q * np * es};
+  const cuuint32_t box[5] = {(cuuint32_t)(kTileX[tile] + 2 * (16 / es)), (cuuint32_t)(kTileY[tile] + 2), 1, 1, 2};
+  const cuuint32_t unit[5] = {1, 1, 1, 1, 1};
+  const CUresult r = encode(m, type, 5, const_cast<void*>(pop), dims, strides, box, unit, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                            CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  if (r != CUDA_SUCCESS) return fail(SC_ECUDA, "cuTensorMapEncodeTiled failed: %d", (int)r);
+  return SC_OK;
+}
 
 // Plans the persistent grid (every resident CTA slot, at most the handle's
 // evaporated-mass slots) and its chunk-major work list: z is cut into nch
-// chunks, item i = (chunk i / cols, column i % cols), CTA b taking items b,
-// b + G, ...; in each round the resident CTAs work on neighbouring columns of
-// the same chunk in lock-step, so a column's halo and shifted-pull sectors come
-// from L2 for its neighbours. Chunks alternate their marching direction. The
-// chunk count trades rounds (ceil(items / G)) against the two halo planes each
-// item stages; zchunk > 0 fixes the chunk length instead.
+// chunks, item i = (chunk i / cols, column i % cols). Chunks alternate their marching
+// direction. The chunk count trades rounds (ceil(items / G)) against the two halo planes
+// each item stages; zchunk > 0 fixes the chunk length instead.
 int plan_launch(const sc_params* p, const Layout& l, int tile, int zchunk, LaunchCfg* c) {
   int dev = 0, sms = 1;
   CK(cudaGetDevice(&dev));
   CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  const int occ = step_ops(p->storage, tile, l.rows).occupancy();
+  const int occ = step_ops(p->storage, tile, l.rows).occupancy(make_dev(p, l));
   if (occ < 1) return fail(SC_ECUDA, "the step kernel cannot be made resident: %s", cudaGetErrorString(cudaGetLastError()));
   c->tile = tile;
   c->cols_x = (p->nx + kTileX[tile] - 1) / kTileX[tile];
@@ -1044,26 +1083,25 @@ int plan_launch(const sc_params* p, const Layout& l, int tile, int zchunk, Launc
   if (n > l.cap_items) return fail(SC_EINVAL, "work list exceeds its capacity");
   c->grid = (int)std::max(1LL, std::min<long long>(slots, n));
   c->items.clear();
-  c->starts.clear();
   c->zmax = 0;
-  for (long long b = 0; b < c->grid; ++b) {
-    c->starts.push_back((int)c->items.size());
-    for (long long it = b; it < n; it += c->grid) {
-      const long long k = it / cols, col = it - k * cols;
-      const int zb = (int)(k * nz / best_nch), ze = (int)((k + 1) * nz / best_nch);
-      c->items.push_back(make_int4((int)col, zb, ze, (int)(k & 1)));
-      c->zmax = std::max(c->zmax, ze - zb);
-    }
+  for (long long it = 0; it < n; ++it) {
+    const long long k = it / cols, col = it - k * cols;
+    const int zb = (int)(k * nz / best_nch), ze = (int)((k + 1) * nz / best_nch);
+    c->items.push_back(make_int4((int)col, zb, ze, (int)(k & 1)));
+    c->zmax = std::max(c->zmax, ze - zb);
   }
-  c->starts.push_back((int)c->items.size());
   return SC_OK;
 }
 
 // Makes c the handle's configuration and uploads its work list (synchronous).
 int apply_launch(sc_lbm* h, const LaunchCfg& c) {
   CK(cudaMemcpyAsync(h->items(), c.items.data(), sizeof(int4) * c.items.size(), cudaMemcpyHostToDevice, h->stream));
-  CK(cudaMemcpyAsync(h->starts(), c.starts.data(), sizeof(int) * c.starts.size(), cudaMemcpyHostToDevice, h->stream));
   CK(cudaStreamSynchronize(h->stream));
+  if (h->lay.rows)
+    for (int k = 0; k < 2; ++k) {
+      const int rc = encode_map(h, h->pop(k), c.tile, &h->maps[k]);
+      if (rc) return rc;
+    }
   h->lay.tile = c.tile;
   h->lay.tx = kTileX[c.tile];
   h->lay.ty = kTileY[c.tile];
@@ -1071,6 +1109,7 @@ int apply_launch(sc_lbm* h, const LaunchCfg& c) {
   h->lay.cols = c.cols;
   h->zmax = c.zmax;
   h->grid = c.grid;
+  h->nitems = (int)c.items.size();
   return SC_OK;
 }
 
@@ -1300,9 +1339,11 @@ int launch_persist(sc_lbm* h, int K, cudaStream_t st) {
   return SC_OK;
 }
 
-// The error word of the persistent step: SC_ETIMEOUT when one of its waits gave up
-// (the lattice's state is then undefined until it is loaded again).
+// After the stream is synchronised: SC_ETIMEOUT when a wait of the persistent step or of a
+// step's plane copies gave up (the lattice's state is then undefined until it is loaded again).
 int persist_status(sc_lbm* h) {
+  if (*(volatile int*)h->h_err != 0)
+    return fail(SC_ETIMEOUT, "a step's copies of a plane did not land in time; load a state to continue");
   if (!h->persist) return SC_OK;
   int v = 0;
   CK(cudaMemcpyAsync(&v, h->err(), sizeof(int), cudaMemcpyDeviceToHost, h->stream));
@@ -1327,7 +1368,8 @@ int launch_one(sc_lbm* h, cudaStream_t st) {
     return SC_OK;
   }
   const int src = h->cur, dst = 1 - h->cur;
-  StepArgs a{h->L, h->pop(src), h->pop(dst), h->evap(), h->lay.cols_x, h->items(), h->starts(), h->grid, st};
+  StepArgs a{h->L, h->pop(src), h->pop(dst), h->evap(), (int)h->lay.nslots, h->lay.cols_x, h->items(), h->nitems,
+             h->next(), h->grid, st, h->maps[src], h->h_err};
   cudaError_t e = step_ops(h->p.storage, h->lay.tile, h->lay.rows).launch(a);
   if (e != cudaSuccess) return fail(SC_ECUDA, "step launch failed: %s", cudaGetErrorString(e));
   h->cur = dst;
@@ -1370,6 +1412,10 @@ int load(sc_lbm* h, long long s0, long long s1, int mode, const float* f, long l
   // every caller loads the whole lattice; in place it is written in the even form
   // (the two-lattice pull's slots); a new state clears the persistent step's error
   if (h->lay.aa) h->cur = 0;
+  if (*(volatile int*)h->h_err != 0) {
+    CK(cudaStreamSynchronize(h->stream));
+    *h->h_err = 0;
+  }
   if (h->persist) CK(cudaMemsetAsync(h->err(), 0, sizeof(int), h->stream));
   switch (h->p.storage) {
     case SC_STORAGE_F16: return launch_load<StF16>(h, s0, s1, mode, f, fs, rho, rs, sh);
@@ -1538,12 +1584,16 @@ static int create_common(const sc_params* p, void* stream, void* buf, bool owns,
     sc_lbm_destroy(h);
     return rc0;
   }
-  cudaError_t e = cudaMallocHost((void**)&h->h_diag, sizeof(double) * p->nz * h->lay.diag_nsplit * kDiagFields);
-  if (e == cudaSuccess) e = cudaMallocHost((void**)&h->h_evap, sizeof(double) * h->lay.nslots);
+  // one pinned block: the diagnostics' partial sums, the evaporated-mass slots, the error word
+  const size_t nd = (size_t)p->nz * h->lay.diag_nsplit * kDiagFields;
+  cudaError_t e = cudaMallocHost((void**)&h->h_diag, sizeof(double) * (nd + h->lay.nslots + 1));
   if (e != cudaSuccess) {
     sc_lbm_destroy(h);
     return fail(SC_ENOMEM, "pinned host allocation failed: %s", cudaGetErrorString(e));
   }
+  h->h_evap = h->h_diag + nd;
+  h->h_err = (int*)(h->h_evap + h->lay.nslots);
+  *h->h_err = 0;
   e = cudaMemsetAsync(buf, 0, h->lay.off_stage, h->stream);
   if (e == cudaSuccess)
     e = cudaMemsetAsync((char*)buf + h->lay.off_flags, 0, h->lay.total - h->lay.off_flags, h->stream);
@@ -1583,7 +1633,6 @@ void sc_lbm_destroy(sc_lbm* h) {
   cudaStreamSynchronize(h->stream);
   if (h->graph) cudaGraphExecDestroy(h->graph);
   if (h->h_diag) cudaFreeHost(h->h_diag);
-  if (h->h_evap) cudaFreeHost(h->h_evap);
   if (h->owns && h->base) cudaFree(h->base);
   delete h;
 }
@@ -1885,7 +1934,7 @@ int sc_lbm_diagnostics_noalloc(sc_lbm* h, double* out_dev) {
   if (rc) return rc;
   k_diag_finish<<<1, 1, 0, h->stream>>>(part, h->p.nz, h->lay.diag_nsplit, (double)h->p.nx * h->p.ny, h->L.wall_z0,
                                         h->L.wall_z1, h->evap(), h->lay.nslots, h->evap_offset,
-                                        h->persist ? h->err() : nullptr, out_dev);
+                                        h->persist ? h->err() : h->h_err, out_dev);
   CK(cudaGetLastError());
   return SC_OK;
 }
@@ -1912,7 +1961,7 @@ int sc_lbm_tune(sc_lbm* h, int32_t trials, int32_t* tile, int32_t* zchunk) {
   // trial launches book their evaporated mass in the read-out staging area and
   // use the handle's work-list buffer; the chosen list is uploaded at the end
   double* scratch = (double*)h->stage();
-  const long long scratch_slots = h->lay.stage_n;  // 2 * stage_n floats
+  const int scratch_slots = (int)std::min(h->lay.nslots, h->lay.stage_n);  // of 2 * stage_n floats
   LaunchCfg best;
   int rc = plan_launch(&h->p, h->lay, h->lay.tile, h->p.zchunk, &best);  // the current choice
   if (rc) return rc;
@@ -1925,10 +1974,10 @@ int sc_lbm_tune(sc_lbm* h, int32_t trials, int32_t* tile, int32_t* zchunk) {
   for (int t = 0; t < kNumTiles && rc == SC_OK; ++t)
     for (int zc : kZc) {
       LaunchCfg c;
-      if (plan_launch(&h->p, h->lay, t, zc, &c) != SC_OK || c.grid > scratch_slots) continue;
+      if (plan_launch(&h->p, h->lay, t, zc, &c) != SC_OK) continue;
       bool dup = false;
       for (const LaunchCfg& o : tried)
-        dup = dup || (o.tile == c.tile && o.grid == c.grid && o.starts == c.starts && o.items.size() == c.items.size() &&
+        dup = dup || (o.tile == c.tile && o.grid == c.grid && o.items.size() == c.items.size() &&
                       std::equal(o.items.begin(), o.items.end(), c.items.begin(), [](const int4& u, const int4& v) {
                         return u.x == v.x && u.y == v.y && u.z == v.z && u.w == v.w;
                       }));
@@ -1936,10 +1985,9 @@ int sc_lbm_tune(sc_lbm* h, int32_t trials, int32_t* tile, int32_t* zchunk) {
       tried.push_back(c);
       cudaError_t e = cudaMemcpyAsync(h->items(), c.items.data(), sizeof(int4) * c.items.size(), cudaMemcpyHostToDevice,
                                       h->stream);
-      if (e == cudaSuccess)
-        e = cudaMemcpyAsync(h->starts(), c.starts.data(), sizeof(int) * c.starts.size(), cudaMemcpyHostToDevice,
-                            h->stream);
-      StepArgs a{h->L, h->pop(h->cur), h->pop(1 - h->cur), scratch, c.cols_x, h->items(), h->starts(), c.grid, h->stream};
+      StepArgs a{h->L, h->pop(h->cur), h->pop(1 - h->cur), scratch, scratch_slots, c.cols_x, h->items(),
+                 (int)c.items.size(), h->next(), c.grid, h->stream, {}, h->h_err};
+      if (h->lay.rows && encode_map(h, h->pop(h->cur), t, &a.map) != SC_OK) e = cudaErrorUnknown;
       const StepOps ops = step_ops(h->p.storage, t, h->lay.rows);
       if (e == cudaSuccess) e = ops.launch(a);  // warm-up
       if (e == cudaSuccess) e = cudaEventRecord(e0, h->stream);

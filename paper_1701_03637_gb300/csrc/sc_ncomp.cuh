@@ -12,7 +12,7 @@
 // the pulled populations into a shared ring of 4 planes, then pulling plane p again
 // (an L2 hit), forming every component's force from the ring, the common velocity
 // and the shifted relaxation, and storing f*. The per-component arithmetic is the
-// two-component kernels' (sum19, psi_of, momentum, force_sum_one = force_sums per
+// two-component kernels' (sum19, psi_of, momentum, force_sums per
 // component, relax_core), and the sums over components are ordered so that two
 // components give their bits.
 
@@ -106,7 +106,7 @@ __device__ __forceinline__ void n_collide_site(const NDev& D, const float* __res
 #pragma unroll
   for (int c = 0; c < NC; ++c) {
     auto psi1 = [&](int sl, int yy, int xx) { return r.v[sl][c][yy + 1][xx + 1]; };
-    force_sum_one(psi1, (p - 1) & 3, p & 3, (p + 1) & 3, ty, tx, a[c]);
+    force_sums(psi1, (p - 1) & 3, p & 3, (p + 1) & 3, ty, tx, a[c]);
   }
 #pragma unroll
   for (int c = 0; c < NC; ++c) {

@@ -97,6 +97,7 @@ struct LatDev {
   double rhoH_mass;        // exact sum of the reset r populations fl(w_i rho_H)
   int geometry, sink_z0, sink_layers;  // sink_z0 in [0, nz)
   double scx, scy, scz, RH2;
+  float sc32[3], RH2_32, r2_tol;       // the sphere in FP32, and the error bound of FP32 r^2 - RH2
   int wall_z0, wall_z1;    // solid slab [wall_z0, wall_z1)
   // z-slab of a larger lattice: local plane z is plane (z + zoff) mod nzg of the lattice
   // whose geometry (sinks, walls, sphere) these fields describe; planes [own0, own1) are
@@ -316,6 +317,13 @@ __device__ __forceinline__ int site_class(const LatDev& L, int x, int y, int zl)
     return (dz < 0 ? dz + L.nzg : dz) < L.sink_layers ? SINK : FLUID;
   }
   if (L.geometry == 2) {
+    // FP32 first: only sites within the error bound of the sphere (72 u X^2 + u RH2, X the
+    // largest extent or centre coordinate, u = 2^-24; a shell 0.01 sites thick at 256^3)
+    // need the FP64 distance, which runs at 1/64 of the FP32 rate (256^3 step with the
+    // sphere: 1.32 ms with FP64 at every site and halo site, 0.99 ms)
+    const float fx = (float)x - L.sc32[0], fy = (float)y - L.sc32[1], fz = (float)z - L.sc32[2];
+    const float far = fx * fx + fy * fy + fz * fz - L.RH2_32;
+    if (fabsf(far) > L.r2_tol) return far > 0.0f ? SINK : FLUID;
     const double dx = (double)x - L.scx, dy = (double)y - L.scy, dz = (double)z - L.scz;
     const double r2 = __dadd_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)), __dmul_rn(dz, dz));
     return r2 >= L.RH2 ? SINK : FLUID;

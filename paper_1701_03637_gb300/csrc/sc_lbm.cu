@@ -953,6 +953,13 @@ LatDev make_dev(const sc_params* p, const Layout& l) {
   for (int i = 0; i < Q; ++i) L.rhoH_mass += (double)(wgt(i) * (float)p->rho_H);
   L.geometry = p->geometry;
   L.sink_z0 = wrap_host(p->sink_z0, p->nz); L.sink_layers = p->sink_layers;
+  {
+    const double X = std::max({std::fabs(p->sphere_cx), std::fabs(p->sphere_cy), std::fabs(p->sphere_cz),
+                               (double)p->nx, (double)p->ny, (double)p->nz});
+    L.sc32[0] = (float)p->sphere_cx; L.sc32[1] = (float)p->sphere_cy; L.sc32[2] = (float)p->sphere_cz;
+    L.RH2_32 = (float)(p->R_H * p->R_H);
+    L.r2_tol = (float)(6e-6 * X * X + 1.2e-7 * p->R_H * p->R_H);
+  }
   L.scx = p->sphere_cx; L.scy = p->sphere_cy; L.scz = p->sphere_cz; L.RH2 = p->R_H * p->R_H;
   if (p->wall_thickness > 0) { L.wall_z0 = p->wall_z0; L.wall_z1 = p->wall_z0 + p->wall_thickness; }
   else { L.wall_z0 = 0; L.wall_z1 = 0; }
@@ -2043,6 +2050,7 @@ int sc_slab_create(const sc_params* g, int32_t z0, int32_t z1, void* stream, sc_
   h->L.wall_z1 = G.wall_z1;
   h->L.sink_z0 = G.sink_z0;
   h->L.sink_layers = G.sink_layers;
+  h->L.r2_tol = G.r2_tol;  // its z runs over the whole lattice
   h->L.nzg = g->nz;
   h->L.zoff = ((z0 - kSlabGhosts) % g->nz + g->nz) % g->nz;
   h->L.own0 = kSlabGhosts;

@@ -1002,6 +1002,7 @@ struct sc_lbm {
   bool slab;                 // z-slab of a larger lattice (sc_slab_create)
   int zmax;  // planes of the longest work item
   int nitems;  // work items of a step (two lattices)
+  int rcta, rsites;  // resident step: CTAs of its cluster (0: not used) and sites of each
   cudaGraphExec_t graph;
   int graph_len;
   int graph_cur;
@@ -1017,6 +1018,8 @@ struct sc_lbm {
   unsigned* next() const { return (unsigned*)(err() + 16); }
   int* err() const { return (int*)(base + lay.off_flags + 2 * kMaxCtas * sizeof(unsigned long long)); }
 };
+
+#include "sc_resident.cuh"
 
 namespace {
 
@@ -1586,6 +1589,7 @@ static int create_common(const sc_params* p, void* stream, void* buf, bool owns,
     LaunchCfg cfg;
     rc0 = plan_launch(p, h->lay, h->lay.tile, p->zchunk, &cfg);
     if (!rc0) rc0 = apply_launch(h, cfg);
+    if (!rc0) plan_resident(h);
   }
   if (rc0) {
     sc_lbm_destroy(h);
@@ -1732,6 +1736,12 @@ int sc_lbm_step(sc_lbm* h, int64_t nsteps) {
     h->step += nsteps;
     return SC_OK;
   }
+  if (h->rcta > 0) {
+    int rc = launch_resident(h, nsteps);
+    if (rc) return rc;
+    h->step += nsteps;
+    return SC_OK;
+  }
   if (left >= 4) {
     int rc = ensure_graph(h);
     if (rc) return rc;
@@ -1752,12 +1762,8 @@ int sc_lbm_step(sc_lbm* h, int64_t nsteps) {
 
 int sc_lbm_read_fields_device(sc_lbm* h, float* rr, float* rb) {
   if (!h || !rr || !rb) return fail(SC_EINVAL, "NULL argument");
-  int rc = canonical(h, 0, h->lay.nsites, h->stage(), h->lay.stage_n, nullptr, 0);
-  if (rc) return rc;
-  CK(cudaMemcpyAsync(rr, h->stage(), sizeof(float) * h->lay.nsites, cudaMemcpyDeviceToDevice, h->stream));
-  CK(cudaMemcpyAsync(rb, h->stage() + h->lay.stage_n, sizeof(float) * h->lay.nsites, cudaMemcpyDeviceToDevice,
-                     h->stream));
-  return SC_OK;
+  // the kernel writes the caller's arrays (rho^b at their distance from rho^r)
+  return canonical(h, 0, h->lay.nsites, rr, rb - rr, nullptr, 0);
 }
 
 int sc_lbm_read_fields(sc_lbm* h, float* rr, float* rb) {
@@ -2056,6 +2062,7 @@ int sc_slab_create(const sc_params* g, int32_t z0, int32_t z1, void* stream, sc_
   h->L.own0 = kSlabGhosts;
   h->L.own1 = kSlabGhosts + (z1 - z0);
   h->slab = true;
+  h->rcta = 0;  // ghost planes are exchanged every step
   *out = h;
   return SC_OK;
 }
@@ -2102,6 +2109,7 @@ int sc_lbm_launch_count(sc_lbm* h, int64_t nsteps, int64_t* launches) {
   if (!h || !launches) return fail(SC_EINVAL, "NULL argument");
   if (nsteps < 0) return fail(SC_EINVAL, "nsteps must be >= 0");
   if (h->persist) *launches = (nsteps + persist_max_steps(h) - 1) / persist_max_steps(h);
+  else if (h->rcta > 0) *launches = (nsteps + kResidentMaxSteps - 1) / kResidentMaxSteps;
   else *launches = h->lay.aa ? 2 * nsteps : nsteps;
   return SC_OK;
 }
@@ -2110,6 +2118,7 @@ const char* sc_lbm_kernel_name(sc_lbm* h) {
   if (!h) return "";
   if (h->persist) return "k_aa_persist (cooperative; up to 1024 steps per launch)";
   if (h->lay.aa) return "k_aa_psi + k_aa_collide";
+  if (h->rcta > 0) return "k_resident (one cluster; up to 4096 steps per launch)";
   return h->lay.rows ? "k_step (staged rows)" : "k_step (per-thread pulls)";
 }
 

@@ -96,8 +96,19 @@ extern "C" {
                                    FP32 site update) or two launches per step (SC_STAGING_THREAD:
                                    Psi of every site into an FP32 (Psi^r, Psi^b) array, 8 bytes
                                    per site, then stream + sink + force + collision in place;
-                                   472 bytes). Results are bit-identical to
-                                   SC_LAYOUT_TWO_LATTICE. Not for batch members. */
+                                   472 bytes). With SC_STAGING_AUTO, tall lattices of large
+                                   planes (nx a multiple of 16 bytes of populations, 384
+                                   tiles of 64 x 4 sites per plane or more, and enough planes
+                                   that the Psi array's memory holds at least 12 of them) take
+                                   neither form: the lattice lies where the two-lattice step
+                                   would keep it and is moved by some planes, alternately down
+                                   and up, through storage that has the Psi array's memory as
+                                   spare planes; each step reads and writes it once, and items
+                                   wait, with a time limit, until their neighbours have read
+                                   what they overwrite. sc_lbm_persist_bands hands such a
+                                   lattice of 2^17 sites per plane or more to the persistent
+                                   step. Results are bit-identical to SC_LAYOUT_TWO_LATTICE.
+                                   Not for batch members. */
 
 /* Physical and geometric parameters of one lattice (Sec. II; geometry of Sec. III). */
 typedef struct sc_params {

@@ -18,7 +18,7 @@ INCLUDE = os.path.join(ROOT, "include")
 BUILD_DIR = os.path.join(PKG, "_build")
 LIB_PATH = os.path.join(BUILD_DIR, "libsc_lbm.so")
 SOURCES = ["sc_lbm.cu"]
-HEADERS = ["sc_kernels.cuh", "sc_resident.cuh", "sc_batch.cuh", "sc_ncomp.cuh"]
+HEADERS = ["sc_kernels.cuh", "sc_resident.cuh", "sc_shift.cuh", "sc_batch.cuh", "sc_ncomp.cuh"]
 ARCH = "-gencode=arch=compute_103a,code=sm_103a"
 
 _lock = threading.Lock()

@@ -26,6 +26,7 @@ namespace sclbm {
 
 constexpr int Q = 19;
 constexpr int FLUID = 0, SINK = 1, SOLID = 2;
+constexpr int kGhosts = 2;  // copied planes on each side of a shifted lattice
 
 // D3Q19, own order: rest, +-x, +-y, +-z, then the 12 face diagonals in
 // opposite pairs (i odd, i+1) with e_{i+1} = -e_i.
@@ -812,9 +813,14 @@ struct Tile {
 //
 // Per plane: wait for the copies, read out plane p (Psi to the ring, own populations
 // to registers), barrier, start plane p + d's copies, collide plane p - d.
-template <int TX, int TY, class S>
+//
+// Shift: the step of a lattice in its own storage, shifted by some planes (k_shift). Two
+// copied planes past the end of the march stand in for the planes across the periodic seam,
+// which the march has overwritten by the time it gets there.
+template <int TX, int TY, class S, bool Shift = false>
 struct TileRows {
   using T = typename S::T;
+  using Index = std::conditional_t<Shift, long long, uint32_t>;  // of a site; copied planes may lie below plane 0
   static constexpr int E = 16 / (int)sizeof(T);           // populations per 16 bytes
   static constexpr int NT = TX * TY, NW = NT / 32, RW = TX + 2, RH = TY + 2, NH = 2 * TX + 2 * RH;
   static constexpr int SW = TX + 2 * E;                   // staged row width
@@ -848,7 +854,7 @@ struct TileRows {
   int tw, th;                  // the tile's sites in x and y
   bool left, right, low, high; // margins and edge rows that come through the side buffer
   unsigned parity;             // of the plane in flight
-  bool active, has_halo;
+  bool active, has_halo, downward;
   double evap;
 
   __device__ __forceinline__ TileRows(const LatDev& L_, Smem& sm_, const T* s_, T* d_, const CUtensorMap* m_)
@@ -858,6 +864,13 @@ struct TileRows {
   }
 
   __device__ __forceinline__ int wrapz(int z) const { return z < 0 ? z + L.nz : (z >= L.nz ? z - L.nz : z); }
+  // Plane of the source buffer that plane zp - dz is read from (zp: near_plane of the march's).
+  __device__ __forceinline__ int near_plane(int p) const { return Shift ? p : wrapz(p); }
+  __device__ __forceinline__ int source_plane(int zp, int dz) const {
+    const int z = zp - dz;
+    if constexpr (Shift) return downward ? (z >= L.nz ? z - L.nz : z) : (z < 0 ? z + L.nz : z);
+    return wrapz(z);
+  }
 
   __device__ __forceinline__ void setup(int bx, int by) {
     const int tid = threadIdx.x;
@@ -905,7 +918,7 @@ struct TileRows {
   }
   __device__ __forceinline__ T* staged_row(int i, int c, int r) { return sm.stage + i * IS + (c * RH + r) * SW; }
   __device__ __forceinline__ const T* source_row(int i, int c, int r, int zp) const {
-    const int zs = wrapz(zp - dir_z_rt(i)), ys = wrap_near(y0 - 1 + r - dir_y_rt(i), L.ny);
+    const int zs = source_plane(zp, dir_z_rt(i)), ys = wrap_near(y0 - 1 + r - dir_y_rt(i), L.ny);
     return src + ((long long)(c * Q + i) * L.np + (long long)zs * L.nxny + (long long)ys * L.nx);
   }
   // This thread's wrapped pieces of plane zp: fetch them into the side buffer, or move
@@ -945,11 +958,12 @@ struct TileRows {
   // Start the copies of plane p (p in [-1, nz]). Box i is issued by lane i / NW of warp
   // i % NW, so no warp issues more than a few.
   __device__ __forceinline__ void issue(int p) {
-    const int zp = wrapz(p);
+    const int zp = near_plane(p);
     if (threadIdx.x == 0) mbar_expect(&sm.bar, (unsigned)(Q * BOX * (int)sizeof(T)));
     const int i = (int)(threadIdx.x / 32) + NW * (int)(threadIdx.x % 32);
     if (i < Q)
-      tma_load5(sm.stage + i * IS, map, x0 - E, y0 - 1 - dir_y_rt(i), wrapz(zp - dir_z_rt(i)), i, 0, &sm.bar);
+      tma_load5(sm.stage + i * IS, map, x0 - E, y0 - 1 - dir_y_rt(i),
+                source_plane(zp, dir_z_rt(i)) + (Shift ? kGhosts : 0), i, 0, &sm.bar);
     side_pieces<true>(zp);
     cp_async_commit();
   }
@@ -958,7 +972,7 @@ struct TileRows {
     const bool ok = mbar_wait(&sm.bar, parity);
     parity ^= 1u;
     cp_async_wait_all();
-    side_pieces<false>(wrapz(p));
+    side_pieces<false>(near_plane(p));
     // the next boxes overwrite what these stores wrote
     asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
     __syncthreads();
@@ -974,7 +988,7 @@ struct TileRows {
     return Pair<S>::cv(q[0], q[RH * SW], wgt(I));
   }
   template <int I>
-  __device__ __forceinline__ float2 pulled(int ly, int lx, bool sol_m, bool sol_p, uint32_t s) const {
+  __device__ __forceinline__ float2 pulled(int ly, int lx, bool sol_m, bool sol_p, Index s) const {
     constexpr int ez = dir_z(I);
     if (ez != 0 && (ez > 0 ? sol_m : sol_p)) {
       const T* p = src + (long long)opp(I) * L.np + s;
@@ -1001,7 +1015,7 @@ struct TileRows {
           f[I] = staged<I>(ty, tx);
         });
       } else {
-        const uint32_t s = (uint32_t)(x + L.nx * y) + (uint32_t)L.nxny * (uint32_t)zp;
+        const Index s = (Index)(x + L.nx * y) + (Index)L.nxny * (Index)source_plane(near_plane(p), 0);
         Unroll<0, Q>::run([&](auto ic) {
           constexpr int I = decltype(ic)::value;
           f[I] = pulled<I>(ty, tx, sol_m, sol_p, s);
@@ -1024,7 +1038,7 @@ struct TileRows {
         if (!walls) {
           hrho = sum19_of<float2>([&](auto ic) { return staged<decltype(ic)::value>(hly, hlx); });
         } else {
-          const uint32_t s = (uint32_t)(hx + L.nx * hy) + (uint32_t)L.nxny * (uint32_t)zp;
+          const Index s = (Index)(hx + L.nx * hy) + (Index)L.nxny * (Index)source_plane(near_plane(p), 0);
           hrho = sum19_of<float2>([&](auto ic) { return pulled<decltype(ic)::value>(hly, hlx, sol_m, sol_p, s); });
         }
         if (hcl == SINK) sink_densities(L, hrho);
@@ -1059,6 +1073,7 @@ struct TileRows {
     const int d = down ? -1 : 1;
     const int first = down ? ze - 1 : zb;
     const int n = ze - zb;
+    downward = down;
     issue(first - d);
     for (int o = 0; o < n + 2; ++o) {
       const int p = first + (o - 1) * d;

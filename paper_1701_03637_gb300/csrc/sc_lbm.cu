@@ -848,7 +848,9 @@ size_t elem_size(int storage) { return storage == SC_STORAGE_F32 ? 4 : 2; }
 struct Layout {
   int tile, tx, ty, cols_x, cols;
   bool rows;                  // staged-rows step kernel (nx a multiple of a 16-byte chunk)
-  bool aa;                    // one population lattice updated in place (SC_LAYOUT_AA)
+  bool aa;                    // one population lattice in the AA forms (SC_LAYOUT_AA)
+  bool shift;                 // one population lattice, shifted by `planes` planes each step (SC_LAYOUT_AA)
+  int planes;
   int aa_segs;                // row segments of kAAThreads sites per row (in place)
   long long aa_units;         // row segments of the lattice (in place)
   long long np;               // array stride (elements)
@@ -864,6 +866,8 @@ int auto_tile(const sc_params* p) {
   if (p->nx >= 16) return 2;
   return 3;
 }
+
+int shift_planes(const sc_params* p, long long es, long long bytes, long long* np);
 
 Layout make_layout(const sc_params* p) {
   Layout l{};
@@ -896,6 +900,16 @@ Layout make_layout(const sc_params* p) {
   l.off_psi = off;
   if (l.aa) off += align256((size_t)l.np * sizeof(float2));  // (Psi^r, Psi^b) per site
   else { l.off_pop[1] = off; off += pop; }
+  // the shifted step takes both regions as planes of the 38 arrays
+  l.planes = shift_planes(p, es, (long long)off, &l.np);
+  if (l.planes > 0) {
+    l.aa = false;
+    l.shift = l.rows = true;
+    const size_t plane = (size_t)p->nx * p->ny * es;
+    l.off_pop[0] = kGhosts * plane;
+    l.off_pop[1] = (kGhosts + l.planes) * plane;
+    l.off_psi = off;
+  }
   l.off_stage = off; off += align256((size_t)2 * l.stage_n * sizeof(float));
   l.off_evap = off; off += align256((size_t)l.nslots * sizeof(double));
   l.off_diag = off; off += align256((size_t)p->nz * l.diag_nsplit * kDiagFields * sizeof(double));
@@ -1030,7 +1044,8 @@ struct LaunchCfg {
   std::vector<int4> items;  // tile column, first plane, end plane, downward
 };
 
-// Tensor map of a population buffer for the staged rows of a tile shape: dimensions
+// Tensor map of a population buffer for the staged rows of a tile shape (a shifted lattice's
+// starts at the copied planes below plane 0 and covers those above too): dimensions
 // (x, y, z, direction, component), a box of one direction's TX + 2 E columns and TY + 2
 // rows of one plane, both components.
 using EncodeFn = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
@@ -1052,7 +1067,7 @@ int encode_map(const sc_lbm* h, const void* pop, int tile, CUtensorMap* m) {
                                  : h->p.storage == SC_STORAGE_BF16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16
                                                                    : CU_TENSOR_MAP_DATA_TYPE_FLOAT16;
   const cuuint64_t nx = h->p.nx, ny = h->p.ny, np = h->lay.np;
-  const cuuint64_t dims[5] = {nx, ny, (cuuint64_t)h->p.nz, Q, 2};
+  const cuuint64_t dims[5] = {nx, ny, (cuuint64_t)(h->p.nz + (h->lay.shift ? 2 * kGhosts : 0)), Q, 2};
   const cuuint64_t strides[4] = {nx * es, nx * ny * es, np * es, Q * np * es};
   const cuuint32_t box[5] = {(cuuint32_t)(kTileX[tile] + 2 * (16 / es)), (cuuint32_t)(kTileY[tile] + 2), 1, 1, 2};
   const cuuint32_t unit[5] = {1, 1, 1, 1, 1};
@@ -1162,6 +1177,8 @@ void apply_persist(sc_lbm* h) {
   if (h->withhold >= h->grid) h->withhold = -1;
 }
 
+bool large_planes(const sc_params* p) { return (long long)p->nx * p->ny >= (1LL << 17); }
+
 // Grids of the in-place step: every resident CTA slot, the collision's at most
 // the evaporated-mass slots.
 int plan_aa(sc_lbm* h) {
@@ -1188,8 +1205,7 @@ int plan_aa(sc_lbm* h) {
   // the persistent step wins where each of its CTAs has a large tile per plane (measured
   // at 512^3: 12.0k against 10.7k MLUPS); on small planes (128^3: 3.8k against 10.6k)
   // the two-pass step is the automatic choice
-  const bool large_planes = (long long)h->p.nx * h->p.ny >= (1LL << 17);
-  if (h->p.staging == SC_STAGING_PERSISTENT || (h->p.staging == SC_STAGING_AUTO && large_planes)) {
+  if (h->p.staging == SC_STAGING_PERSISTENT || (h->p.staging == SC_STAGING_AUTO && large_planes(&h->p))) {
     h->persist = plan_persist(h);
     if (!h->persist && h->p.staging == SC_STAGING_PERSISTENT)
       return fail(SC_EINVAL, "the persistent in-place step is not available here: %s", h->persist_why);
@@ -1364,7 +1380,10 @@ int persist_status(sc_lbm* h) {
   return SC_OK;
 }
 
+int launch_shift_one(sc_lbm* h, cudaStream_t st);
+
 int launch_one(sc_lbm* h, cudaStream_t st) {
+  if (h->lay.shift) return launch_shift_one(h, st);
   if (h->lay.aa) {
     cudaError_t e;
     switch (h->p.storage) {
@@ -1456,6 +1475,12 @@ int reset_counters(sc_lbm* h) {
   h->evap_offset = 0.0;
   return SC_OK;
 }
+
+}  // namespace
+
+#include "sc_shift.cuh"
+
+namespace {
 
 // Sites per slab so a slab's 2*19 FP32 populations fit the staging area.
 long long slab_sites(const sc_lbm* h) { return std::max<long long>(1, (2 * h->lay.stage_n) / (2 * Q)); }
@@ -1585,6 +1610,8 @@ static int create_common(const sc_params* p, void* stream, void* buf, bool owns,
   int rc0 = SC_OK;
   if (h->lay.aa) {
     rc0 = plan_aa(h);
+  } else if (h->lay.shift) {
+    rc0 = plan_shift(h);
   } else {
     LaunchCfg cfg;
     rc0 = plan_launch(p, h->lay, h->lay.tile, p->zchunk, &cfg);
@@ -1965,7 +1992,7 @@ int sc_lbm_launch_info(sc_lbm* h, int32_t* tx, int32_t* ty, int32_t* zchunk, int
 int sc_lbm_tune(sc_lbm* h, int32_t trials, int32_t* tile, int32_t* zchunk) {
   Range range("sc_lbm_tune");
   if (!h) return fail(SC_EINVAL, "NULL handle");
-  if (h->lay.aa) {  // one configuration, and no spare buffer for trial launches
+  if (h->lay.aa || h->lay.shift) {  // one configuration, and no spare buffer for trial launches
     if (tile) *tile = 0;
     if (zchunk) *zchunk = h->zmax;
     return SC_OK;
@@ -2110,7 +2137,7 @@ int sc_lbm_launch_count(sc_lbm* h, int64_t nsteps, int64_t* launches) {
   if (nsteps < 0) return fail(SC_EINVAL, "nsteps must be >= 0");
   if (h->persist) *launches = (nsteps + persist_max_steps(h) - 1) / persist_max_steps(h);
   else if (h->rcta > 0) *launches = (nsteps + kResidentMaxSteps - 1) / kResidentMaxSteps;
-  else *launches = h->lay.aa ? 2 * nsteps : nsteps;
+  else *launches = h->lay.aa || h->lay.shift ? 2 * nsteps : nsteps;
   return SC_OK;
 }
 
@@ -2118,6 +2145,7 @@ const char* sc_lbm_kernel_name(sc_lbm* h) {
   if (!h) return "";
   if (h->persist) return "k_aa_persist (cooperative; up to 1024 steps per launch)";
   if (h->lay.aa) return "k_aa_psi + k_aa_collide";
+  if (h->lay.shift) return "k_shift_begin + k_shift (staged rows, one lattice shifted in its storage)";
   if (h->rcta > 0) return "k_resident (one cluster; up to 4096 steps per launch)";
   return h->lay.rows ? "k_step (staged rows)" : "k_step (per-thread pulls)";
 }
@@ -2136,6 +2164,20 @@ int sc_lbm_persist_bands(sc_lbm* h, int32_t request, int32_t* bands) {
   if (!h) return fail(SC_EINVAL, "NULL handle");
   if (request < -1) return fail(SC_EINVAL, "request must be -1, 0 or a band count");
   if (request >= 0) {
+    if (h->lay.shift && large_planes(&h->p)) {  // its persistent plan, where one exists
+      const Layout lay = h->lay;
+      const int cur = h->cur;
+      int rc = shift_to_persist(h);
+      if (rc) return rc;
+      rc = plan_aa(h);
+      if (rc || !h->persist) {
+        h->lay = lay;
+        h->cur = cur;
+        h->persist = false;
+        const int back = plan_shift(h);
+        if (rc || back) return rc ? rc : back;
+      }
+    }
     if (!h->persist) return fail(SC_EINVAL, "the lattice does not use the persistent in-place step");
     if (request > 1 && (h->p.nx % request != 0 || h->p.nx / request < 2))
       return fail(SC_EINVAL, "%d bands must divide nx = %d into bands of at least 2 sites", request, h->p.nx);

@@ -8,7 +8,10 @@
 // tau F / rho velocity shift), writing f*(t) to the other buffer. The canonical
 // (post-stream, post-sink) populations of step t are pull + sink of the buffer.
 //
-// Memory layout: 2 x 19 arrays (component-major, then direction) of np elements;
+// Memory layout: 19 arrays (one per direction) of np pairs (r, b): the populations of both
+// components in one word (float2, or two 16-bit values), so that a load, a store and a copy
+// move both (with an array per component, half the instructions of a pull were address
+// arithmetic and copies: 256^3 FP16 step 0.90 -> 0.80 ms, 151 x 93 x 67 FP32 90 -> 69 us);
 // site s = x + nx (y + ny z) with x fastest, rows contiguous without padding so
 // that neighbouring tiles share every fetched sector through L2. Periodic wrap
 // is index arithmetic.
@@ -116,13 +119,11 @@ __device__ __forceinline__ int global_z(const LatDev& L, int z) {
 __device__ __forceinline__ bool own_z(const LatDev& L, int z) { return z >= L.own0 && z < L.own1; }
 
 // ------------------------------------------------------------------ storage types
-// ld: a population from global memory. pull_async: start a 4-byte asynchronous
-// copy (cp.async, cached in L1) of the word holding a population into shared
-// memory and return which half of the word it is (16-bit types). word: the
-// population from such a word.
-__device__ __forceinline__ void cp_async4(uint32_t* smem, const void* gmem) {
+// Asynchronous copy of a pair (4 or 8 bytes), cached in L1.
+template <int BYTES>
+__device__ __forceinline__ void cp_async_ca(void* smem, const void* gmem) {
   const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(sa), "l"(gmem) : "memory");
+  asm volatile("cp.async.ca.shared.global [%0], [%1], %2;\n" ::"r"(sa), "l"(gmem), "n"(BYTES) : "memory");
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
@@ -158,14 +159,13 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, unsigned parity) {
     if (global_ns() - t0 > 2000000000ull) return false;
   return true;
 }
-// A box of the tensor at element coordinates (x, y, z, i, c); the x start must lie on a
+// A box of the tensor at element coordinates (x, y, z, i); the x start must lie on a
 // 16-byte boundary, parts outside the tensor are filled with zeros.
-__device__ __forceinline__ void tma_load5(void* smem, const CUtensorMap* map, int x, int y, int z, int i, int c,
-                                          uint64_t* bar) {
+__device__ __forceinline__ void tma_load4(void* smem, const CUtensorMap* map, int x, int y, int z, int i, uint64_t* bar) {
   asm volatile(
-      "cp.async.bulk.tensor.5d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5, %6}], "
-      "[%7];\n" ::"r"(smem_addr(smem)),
-      "l"(map), "r"(x), "r"(y), "r"(z), "r"(i), "r"(c), "r"(smem_addr(bar))
+      "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5}], "
+      "[%6];\n" ::"r"(smem_addr(smem)),
+      "l"(map), "r"(x), "r"(y), "r"(z), "r"(i), "r"(smem_addr(bar))
       : "memory");
 }
 // 16-byte asynchronous copy, cached in L2 only; both addresses 16-byte aligned.
@@ -173,118 +173,62 @@ __device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(smem_addr(smem)), "l"(gmem) : "memory");
 }
 
-// ldcg: a population read at L2 only (ld.global.cg), never from L1, for kernels in
-// which other CTAs of the same launch overwrite the data between two reads.
+// T: the stored pair (r, b) of one direction; cv decodes it and enc encodes it (w is the
+// direction's weight), each half with the single population's operations. ld, ldcg: a pair
+// from global memory, ldcg at L2 only (never from L1), for kernels in which other CTAs of the
+// same launch overwrite the data between two reads. put: population stores to global memory
+// are evict-first: the next step reads them only after the whole lattice has gone by, and until
+// then they displace what neighbouring CTAs share in the L2 (256^3 FP32 with the spherical
+// sink: 1.18 against 1.08 ms per step).
 struct StF32 {
-  using T = float;
-  static __device__ __forceinline__ float ld(const T* p, float) { return __ldg(p); }
-  static __device__ __forceinline__ float ldcg(const T* p, float) { return __ldcg(p); }
-  static __device__ __forceinline__ float cv(T v, float) { return v; }
-  static __device__ __forceinline__ T enc(float v, float) { return v; }
-  static __device__ __forceinline__ void put(T* p, T v) { __stcs(p, v); }
-  static __device__ __forceinline__ uint32_t pull_async(uint32_t* sm, const T* p) {
-    cp_async4(sm, p);
-    return 0u;
-  }
-  static __device__ __forceinline__ float word(uint32_t w, uint32_t, float) { return __uint_as_float(w); }
+  using T = float2;
+  static __device__ __forceinline__ float2 cv(T v, float) { return v; }
+  static __device__ __forceinline__ T enc(float2 v, float) { return v; }
 };
-// FP16 / BF16 offsets h = f - w_i * rho0 (rho0 = 1), round to nearest even.
-// Arrays hold an even number of elements, so the aligned word of any element
-// lies inside its array.
-template <class Half>
-__device__ __forceinline__ uint32_t pull_async16(uint32_t* sm, const Half* p) {
-  const uintptr_t a = reinterpret_cast<uintptr_t>(p);
-  cp_async4(sm, reinterpret_cast<const void*>(a & ~uintptr_t(3)));
-  return (uint32_t)(a >> 1) & 1u;
+// FP16 / BF16 offsets h = f - w_i * rho0 (rho0 = 1), round to nearest even; component r in
+// the low half.
+__device__ __forceinline__ float2 half_pair(uint32_t v) {
+  return make_float2(__half2float(__ushort_as_half((unsigned short)(v & 0xffffu))),
+                     __half2float(__ushort_as_half((unsigned short)(v >> 16))));
 }
-__device__ __forceinline__ unsigned short ldcg16(const void* p) {
-  return __ldcg(reinterpret_cast<const unsigned short*>(p));
+__device__ __forceinline__ uint32_t half_word(float2 v) {
+  const __half2 p = __floats2half2_rn(v.x, v.y);
+  return (uint32_t)__half_as_ushort(__low2half(p)) | (uint32_t)__half_as_ushort(__high2half(p)) << 16;
 }
-// Population stores to global memory are evict-first: the next step reads them only after
-// the whole lattice has gone by, and until then they displace what neighbouring CTAs share
-// in the L2 (256^3 FP32 with the spherical sink: 1.18 against 1.08 ms per step).
-__device__ __forceinline__ void put16(void* p, unsigned short v) { __stcs(reinterpret_cast<unsigned short*>(p), v); }
 struct StF16 {
-  using T = __half;
-  static __device__ __forceinline__ float ld(const T* p, float w) { return w + __half2float(__ldg(p)); }
-  static __device__ __forceinline__ float ldcg(const T* p, float w) { return w + __half2float(__ushort_as_half(ldcg16(p))); }
-  static __device__ __forceinline__ float cv(T v, float w) { return w + __half2float(v); }
-  static __device__ __forceinline__ T enc(float v, float w) { return __float2half_rn(v - w); }
-  static __device__ __forceinline__ void put(T* p, T v) { put16(p, __half_as_ushort(v)); }
-  static __device__ __forceinline__ uint32_t pull_async(uint32_t* sm, const T* p) { return pull_async16(sm, p); }
-  static __device__ __forceinline__ float word(uint32_t w, uint32_t hi, float wt) {
-    return wt + __half2float(__ushort_as_half((unsigned short)(hi ? w >> 16 : w & 0xffffu)));
-  }
+  using T = uint32_t;
+  static __device__ __forceinline__ float2 cv(T v, float w) { return vadd(make_float2(w, w), half_pair(v)); }
+  static __device__ __forceinline__ T enc(float2 v, float w) { return half_word(vsub(v, make_float2(w, w))); }
 };
 // FP16 of the population scaled by its weight, g = f_i / w_i (about rho),
 // round to nearest even: the same relative spacing in the liquid and the vapour.
 struct StF16S {
-  using T = __half;
-  static __device__ __forceinline__ float ld(const T* p, float w) { return __fmul_rn(w, __half2float(__ldg(p))); }
-  static __device__ __forceinline__ float ldcg(const T* p, float w) {
-    return __fmul_rn(w, __half2float(__ushort_as_half(ldcg16(p))));
+  using T = uint32_t;
+  // not a packed product: that was contracted into momentum's differences
+  static __device__ __forceinline__ float2 cv(T v, float w) {
+    const float2 h = half_pair(v);
+    return make_float2(__fmul_rn(w, h.x), __fmul_rn(w, h.y));
   }
-  static __device__ __forceinline__ float cv(T v, float w) { return __fmul_rn(w, __half2float(v)); }
   // w is a compile-time weight at every call, so 1 / w folds to a constant
-  static __device__ __forceinline__ T enc(float v, float w) { return __float2half_rn(__fmul_rn(v, 1.0f / w)); }
-  static __device__ __forceinline__ void put(T* p, T v) { put16(p, __half_as_ushort(v)); }
-  static __device__ __forceinline__ uint32_t pull_async(uint32_t* sm, const T* p) { return pull_async16(sm, p); }
-  static __device__ __forceinline__ float word(uint32_t w, uint32_t hi, float wt) {
-    return __fmul_rn(wt, __half2float(__ushort_as_half((unsigned short)(hi ? w >> 16 : w & 0xffffu))));
-  }
+  static __device__ __forceinline__ T enc(float2 v, float w) { return half_word(vmul(v, make_float2(1.0f / w, 1.0f / w))); }
 };
 struct StBF16 {
-  using T = __nv_bfloat16;
-  static __device__ __forceinline__ float ld(const T* p, float w) { return w + __bfloat162float(__ldg(p)); }
-  static __device__ __forceinline__ float ldcg(const T* p, float w) {
-    return w + __bfloat162float(__ushort_as_bfloat16(ldcg16(p)));
+  using T = uint32_t;
+  static __device__ __forceinline__ float2 cv(T v, float w) {  // a bfloat16 is the upper half of its float
+    return vadd(make_float2(w, w), make_float2(__uint_as_float(v << 16), __uint_as_float(v & 0xffff0000u)));
   }
-  static __device__ __forceinline__ float cv(T v, float w) { return w + __bfloat162float(v); }
-  static __device__ __forceinline__ T enc(float v, float w) { return __float2bfloat16_rn(v - w); }
-  static __device__ __forceinline__ void put(T* p, T v) { put16(p, __bfloat16_as_ushort(v)); }
-  static __device__ __forceinline__ uint32_t pull_async(uint32_t* sm, const T* p) { return pull_async16(sm, p); }
-  static __device__ __forceinline__ float word(uint32_t w, uint32_t hi, float wt) {
-    return wt + __bfloat162float(__ushort_as_bfloat16((unsigned short)(hi ? w >> 16 : w & 0xffffu)));
+  static __device__ __forceinline__ T enc(float2 v, float w) {
+    const float2 h = vsub(v, make_float2(w, w));
+    const __nv_bfloat162 p = __floats2bfloat162_rn(h.x, h.y);
+    return (uint32_t)__bfloat16_as_ushort(__low2bfloat16(p)) | (uint32_t)__bfloat16_as_ushort(__high2bfloat16(p)) << 16;
   }
 };
-
-// The pair (r, b) of one direction: decoded from (cv) and encoded to (enc) the storage type
-// with the single population's operations; st: encoded to two arrays in global memory.
 template <class S>
-struct Pair {
-  using T = typename S::T;
-  static __device__ __forceinline__ float2 cv(T r, T b, float w) {
-    if constexpr (std::is_same<S, StF16>::value)
-      return vadd(make_float2(w, w), make_float2(__half2float(r), __half2float(b)));
-    else if constexpr (std::is_same<S, StBF16>::value)
-      return vadd(make_float2(w, w), make_float2(__bfloat162float(r), __bfloat162float(b)));
-    else  // scaled FP16: a packed product by a constant was contracted into momentum's differences
-      return make_float2(S::cv(r, w), S::cv(b, w));
-  }
-  static __device__ __forceinline__ void enc(float2 v, float w, T& r, T& b) {
-    if constexpr (std::is_same<S, StF32>::value) {
-      r = v.x;
-      b = v.y;
-    } else if constexpr (std::is_same<S, StBF16>::value) {
-      const float2 h = vsub(v, make_float2(w, w));
-      const __nv_bfloat162 p = __floats2bfloat162_rn(h.x, h.y);
-      r = __low2bfloat16(p);
-      b = __high2bfloat16(p);
-    } else {
-      const float2 h = std::is_same<S, StF16>::value ? vsub(v, make_float2(w, w))
-                                                     : vmul(v, make_float2(1.0f / w, 1.0f / w));
-      const __half2 p = __floats2half2_rn(h.x, h.y);
-      r = __low2half(p);
-      b = __high2half(p);
-    }
-  }
-  static __device__ __forceinline__ void st(T* pr, T* pb, float2 v, float w) {
-    T r, b;
-    enc(v, w, r, b);
-    S::put(pr, r);
-    S::put(pb, b);
-  }
-};
+__device__ __forceinline__ float2 ld(const typename S::T* p, float w) { return S::cv(__ldg(p), w); }
+template <class S>
+__device__ __forceinline__ float2 ldcg(const typename S::T* p, float w) { return S::cv(__ldcg(p), w); }
+template <class S>
+__device__ __forceinline__ void put(typename S::T* p, float2 v, float w) { __stcs(p, S::enc(v, w)); }
 
 __host__ __device__ __forceinline__ int wrapi(int v, int n) {
   v %= n;
@@ -370,32 +314,24 @@ struct PullIdx {
 template <class S>
 __device__ __forceinline__ void pull_full(const LatDev& L, const typename S::T* __restrict__ src, const PullIdx& P,
                                           float2 (&f)[Q]) {
-  const long long cstride = (long long)Q * L.np;
   Unroll<0, Q>::run([&](auto ic) {
     constexpr int I = decltype(ic)::value;
     int idx, d;
     P.template at<I>(idx, d);
-    const typename S::T* p = src + (long long)d * L.np + idx;
-    f[I] = make_float2(S::ld(p, wgt(I)), S::ld(p + cstride, wgt(I)));
+    f[I] = ld<S>(src + (long long)d * L.np + idx, wgt(I));
   });
 }
 
-// Asynchronous form of pull_full: population (c, i) goes to sm[(c Q + i) stride];
-// bit i of the result says which half of the word holds direction i.
+// Asynchronous form of pull_full: the pair of direction i goes to sm[i stride].
 template <class S>
-__device__ __forceinline__ uint32_t pull_async(const LatDev& L, const typename S::T* __restrict__ src,
-                                               const PullIdx& P, uint32_t* sm, int stride) {
-  const long long cstride = (long long)Q * L.np;
-  uint32_t hi = 0u;
+__device__ __forceinline__ void pull_async(const LatDev& L, const typename S::T* __restrict__ src, const PullIdx& P,
+                                           typename S::T* sm, int stride) {
   Unroll<0, Q>::run([&](auto ic) {
     constexpr int I = decltype(ic)::value;
     int idx, d;
     P.template at<I>(idx, d);
-    const typename S::T* p = src + (long long)d * L.np + idx;
-    hi |= S::pull_async(sm + I * stride, p) << I;
-    S::pull_async(sm + (Q + I) * stride, p + cstride);
+    cp_async_ca<sizeof(typename S::T)>(sm + I * stride, src + (long long)d * L.np + idx);
   });
-  return hi;
 }
 
 // Density from the 19 populations of a site: opposite pairs (I, I+1) first, then
@@ -458,12 +394,8 @@ __device__ __forceinline__ float2 psi_of(float2 rho) { return make_float2(psi_of
 template <class S>
 __device__ __forceinline__ void store_site(const LatDev& L, typename S::T* __restrict__ dst, int s,
                                            const float2 (&f)[Q]) {
-  const long long cstride = (long long)Q * L.np;
 #pragma unroll
-  for (int i = 0; i < Q; ++i) {
-    typename S::T* p = dst + (long long)i * L.np + s;
-    Pair<S>::st(p, p + cstride, f[i], wgt(i));
-  }
+  for (int i = 0; i < Q; ++i) put<S>(dst + (long long)i * L.np + s, f[i], wgt(i));
 }
 
 // Momentum sum_i f_i e_i of each component from the differences of opposite
@@ -619,7 +551,7 @@ __device__ __forceinline__ void force_sums(PsiAt psi, int sm1, int s0, int sp1, 
 // while plane z-2's slot is free.
 //
 // The pulls of the next plane are asynchronous copies into shared slots that
-// belong to the issuing thread alone (its site's 38 populations, and its halo
+// belong to the issuing thread alone (its site's 19 pairs, and its halo
 // site's), started as soon as the current plane has been read out of them, so
 // their latency overlaps the collision of the previous plane without holding
 // registers. Only the thread that issued a copy reads its slot, so a wait on its
@@ -634,8 +566,8 @@ struct Tile {
   struct Smem {
     float2 ring[4][RH][RW];  // (Psi^r, Psi^b) of plane slot, tile row + 1, tile column + 1
     double red[NW];
-    uint32_t fin[2 * Q][NT];       // pulled populations of the own site, [c Q + i][thread]
-    uint32_t fh[2 * Q][HS];        // pulled populations of the halo site, [c Q + i][thread]
+    typename S::T fin[Q][NT];      // pulled pairs of the own site, [i][thread]
+    typename S::T fh[Q][HS];       // pulled pairs of the halo site, [i][thread]
   };
 
   const LatDev& L;
@@ -651,8 +583,8 @@ struct Tile {
       : L(L_), sm(sm_), src(s_), dst(d_), evap(0.0) {}
 
   __device__ __forceinline__ int wrapz(int z) const { return z < 0 ? z + L.nz : (z >= L.nz ? z - L.nz : z); }
-  __device__ __forceinline__ uint32_t* own_slot() { return &sm.fin[0][threadIdx.x]; }
-  __device__ __forceinline__ uint32_t* halo_slot() { return &sm.fh[0][threadIdx.x]; }
+  __device__ __forceinline__ typename S::T* own_slot() { return &sm.fin[0][threadIdx.x]; }
+  __device__ __forceinline__ typename S::T* halo_slot() { return &sm.fh[0][threadIdx.x]; }
 
   // Bind the CTA to tile column (bx, by). Lanes past a ragged edge stage the
   // wrapped site there (its Psi is the halo of the last real site).
@@ -676,32 +608,28 @@ struct Tile {
   }
 
   // Start the pulls of plane p (p in [-1, nz]) for the own site and the halo site.
-  __device__ __forceinline__ void issue(int p, int& cls, uint32_t& hi, int& hcl, uint32_t& hhi) {
+  __device__ __forceinline__ void issue(int p, int& cls, int& hcl) {
     const int zp = wrapz(p);
     cls = site_class(L, x, y, zp);
-    if (cls != SOLID) hi = pull_async<S>(L, src, PullIdx(L, x, y, zp), own_slot(), NT);
+    if (cls != SOLID) pull_async<S>(L, src, PullIdx(L, x, y, zp), own_slot(), NT);
     if (has_halo) {
       hcl = site_class(L, hx, hy, zp);
-      if (hcl != SOLID) hhi = pull_async<S>(L, src, PullIdx(L, hx, hy, zp), halo_slot(), HS);
+      if (hcl != SOLID) pull_async<S>(L, src, PullIdx(L, hx, hy, zp), halo_slot(), HS);
     }
     cp_async_commit();
   }
 
   // Read plane p out of the slots (after the wait): the own site into f, the
   // halo site as sums; apply the sink and publish Psi to ring slot p & 3.
-  __device__ __forceinline__ void take(int p, bool own, int cls, uint32_t hi, int hcl, uint32_t hhi, float2 (&f)[Q],
-                                       float2& rho) {
+  __device__ __forceinline__ void take(int p, bool own, int cls, int hcl, float2 (&f)[Q], float2& rho) {
     const int slot = p & 3;
     float2 ps = make_float2(0.0f, 0.0f);
     if (cls == SOLID) {
       rho = ps;
     } else {
-      const uint32_t* w = own_slot();
+      const typename S::T* w = own_slot();
 #pragma unroll
-      for (int i = 0; i < Q; ++i) {
-        const uint32_t h = (hi >> i) & 1u;
-        f[i] = make_float2(S::word(w[i * NT], h, wgt(i)), S::word(w[(Q + i) * NT], h, wgt(i)));
-      }
+      for (int i = 0; i < Q; ++i) f[i] = S::cv(w[i * NT], wgt(i));
       rho = sum19(f);
       if (cls == SINK) {
         if (active && own && own_z(L, wrapz(p))) evap += (double)sink_excess(L, f);
@@ -713,12 +641,11 @@ struct Tile {
     if (has_halo) {
       float2 hps = make_float2(0.0f, 0.0f);
       if (hcl != SOLID) {
-        const uint32_t* w = halo_slot();
+        const typename S::T* w = halo_slot();
         // the owner's arithmetic, so the halo Psi has the owner's bits
         float2 hrho = sum19_of<float2>([&](auto ic) {
           constexpr int I = decltype(ic)::value;
-          const uint32_t h = (hhi >> I) & 1u;
-          return make_float2(S::word(w[I * HS], h, wgt(I)), S::word(w[(Q + I) * HS], h, wgt(I)));
+          return S::cv(w[I * HS], wgt(I));
         });
         if (hcl == SINK) sink_densities(L, hrho);
         hps = psi_of(hrho);
@@ -754,17 +681,16 @@ struct Tile {
     float2 c[Q], n2[Q];
     float2 crho = make_float2(0.f, 0.f), nrho = crho;
     int ccl = SOLID, ncl = SOLID, hcl = SOLID;
-    uint32_t hi = 0u, hhi = 0u;
     const int d = down ? -1 : 1;
     const int first = down ? ze - 1 : zb;
     const int n = ze - zb;
-    issue(first - d, ncl, hi, hcl, hhi);
+    issue(first - d, ncl, hcl);
     for (int o = 0; o < n + 2; ++o) {
       const int p = first + (o - 1) * d;
       cp_async_wait_all();
-      take(p, o >= 1 && o <= n, ncl, hi, hcl, hhi, n2, nrho);
+      take(p, o >= 1 && o <= n, ncl, hcl, n2, nrho);
       const int pcl = ncl;
-      if (o + 1 < n + 2) issue(p + d, ncl, hi, hcl, hhi);
+      if (o + 1 < n + 2) issue(p + d, ncl, hcl);
       __syncthreads();
       if (o >= 2) finish(p - d, c, crho, ccl);
 #pragma unroll
@@ -795,9 +721,9 @@ struct Tile {
 // The same march as Tile, with the pulls staged cooperatively. For each of the 19
 // directions the plane's source rows -- the TY + 2 rows y0 - 1 .. y0 + TY shifted by
 // -e_y, in plane z - e_z -- are copied into shared memory over columns x0 - E ..
-// x0 + TX + E (E populations are 16 bytes), and the x shift -e_x is applied when a thread
+// x0 + TX + E (E pairs are 16 bytes), and the x shift -e_x is applied when a thread
 // reads them. The E-column margins hold the side halo, so the halo needs no pulls of its
-// own. One direction is one TMA box of both components. Requires nx % E == 0 (then the
+// own. One direction is one TMA box. Requires nx % E == 0 (then the
 // box starts on a 16-byte boundary). A population whose source plane is solid is the
 // site's own opposite population (halfway bounce-back): read directly.
 //
@@ -821,19 +747,19 @@ template <int TX, int TY, class S, bool Shift = false>
 struct TileRows {
   using T = typename S::T;
   using Index = std::conditional_t<Shift, long long, uint32_t>;  // of a site; copied planes may lie below plane 0
-  static constexpr int E = 16 / (int)sizeof(T);           // populations per 16 bytes
+  static constexpr int E = 16 / (int)sizeof(T);           // pairs per 16 bytes
   static constexpr int NT = TX * TY, NW = NT / 32, RW = TX + 2, RH = TY + 2, NH = 2 * TX + 2 * RH;
   static constexpr int SW = TX + 2 * E;                   // staged row width
   static constexpr int CH = SW / E;                       // 16-byte pieces per staged row
-  static constexpr int NR = 2 * Q * RH;                   // staged rows per plane
-  static constexpr int BOX = 2 * RH * SW;                 // populations per box
+  static constexpr int NR = Q * RH;                       // staged rows per plane
+  static constexpr int BOX = RH * SW;                     // pairs per box
   static constexpr int IS = (BOX * (int)sizeof(T) + 127) / 128 * 128 / (int)sizeof(T);  // box stride (128-byte aligned)
-  static constexpr int YR = 38;                           // wrapped rows per y edge: 2 (5 directions x 2 + 9 x 1)
+  static constexpr int YR = 19;                           // wrapped rows per y edge: 5 directions x 2 + 9 x 1
   static_assert(TX % E == 0, "tile width must be a multiple of the chunk");
   static_assert(NH <= NT && NT % 32 == 0, "tile shape");
 
   struct Smem {
-    T stage[Q * IS];         // rows of plane p: [i][c][y - y0 + 1][x - x0 + E], box i at i IS
+    T stage[Q * IS];         // rows of plane p: [i][y - y0 + 1][x - x0 + E], box i at i IS
     float2 ring[4][RH][RW];  // (Psi^r, Psi^b) of plane slot, tile row + 1, tile column + 1
     double red[NW];
     uint64_t bar;            // completes when a plane's boxes have landed
@@ -898,8 +824,7 @@ struct TileRows {
     hy = wrapi(by * TY + hly, L.ny);
   }
 
-  // Wrapped rows of a y edge, k in [0, YR / 2) of component c: direction i and staged row
-  // r. At the low edge the rows of tile rows -1 (e_y >= 0) and 0 (e_y > 0), whose sources
+  // Wrapped rows of a y edge, k in [0, YR): direction i and staged row r. At the low edge the rows of tile rows -1 (e_y >= 0) and 0 (e_y > 0), whose sources
   // lie below row 0; at the high edge those of tile rows th and th - 1.
   __device__ __forceinline__ static void wrapped_row(int k, bool hi_edge, int& i, int& which) {
     // directions with e_y = +1: 3 7 10 15 17, with e_y = -1: 4 8 9 16 18, e_y = 0 the rest
@@ -916,10 +841,10 @@ struct TileRows {
       which = j / 5;
     }
   }
-  __device__ __forceinline__ T* staged_row(int i, int c, int r) { return sm.stage + i * IS + (c * RH + r) * SW; }
-  __device__ __forceinline__ const T* source_row(int i, int c, int r, int zp) const {
+  __device__ __forceinline__ T* staged_row(int i, int r) { return sm.stage + i * IS + r * SW; }
+  __device__ __forceinline__ const T* source_row(int i, int r, int zp) const {
     const int zs = source_plane(zp, dir_z_rt(i)), ys = wrap_near(y0 - 1 + r - dir_y_rt(i), L.ny);
-    return src + ((long long)(c * Q + i) * L.np + (long long)zs * L.nxny + (long long)ys * L.nx);
+    return src + ((long long)i * L.np + (long long)zs * L.nxny + (long long)ys * L.nx);
   }
   // This thread's wrapped pieces of plane zp: fetch them into the side buffer, or move
   // them from there into the staged rows.
@@ -928,27 +853,27 @@ struct TileRows {
     T* side = sm.side;
     for (int e = left ? 0 : 1; e < (right ? 2 : 1); ++e) {
       for (int R = threadIdx.x; R < NR; R += NT) {
-        const int i = R / (2 * RH), cr = R - i * 2 * RH, c = cr / RH, r = cr - c * RH;
+        const int i = R / RH, r = R - i * RH;
         T* piece = side + R * E;
         if (FETCH) {
-          cp_async16(piece, source_row(i, c, r, zp) + (e == 0 ? L.nx - E : wrap_near(x0 + tw, L.nx)));
+          cp_async16(piece, source_row(i, r, zp) + (e == 0 ? L.nx - E : wrap_near(x0 + tw, L.nx)));
         } else {
-          *reinterpret_cast<int4*>(staged_row(i, c, r) + (e == 0 ? 0 : tw + E)) = *reinterpret_cast<const int4*>(piece);
+          *reinterpret_cast<int4*>(staged_row(i, r) + (e == 0 ? 0 : tw + E)) = *reinterpret_cast<const int4*>(piece);
         }
       }
       side += NR * E;
     }
     for (int e = low ? 0 : 1; e < (high ? 2 : 1); ++e) {
       for (int q = threadIdx.x; q < YR * CH; q += NT) {
-        const int row = q / CH, j = q - row * CH, c = row >= YR / 2 ? 1 : 0, k = row - c * (YR / 2);
+        const int k = q / CH, j = q - k * CH;
         int i, which;
         wrapped_row(k, e == 1, i, which);
         const int r = e == 0 ? which : th + 1 - which;
         T* piece = side + q * E;
         if (FETCH) {
-          cp_async16(piece, source_row(i, c, r, zp) + wrap_near(x0 - E + j * E, L.nx));
+          cp_async16(piece, source_row(i, r, zp) + wrap_near(x0 - E + j * E, L.nx));
         } else if (r >= 0 && r < RH) {
-          *reinterpret_cast<int4*>(staged_row(i, c, r) + j * E) = *reinterpret_cast<const int4*>(piece);
+          *reinterpret_cast<int4*>(staged_row(i, r) + j * E) = *reinterpret_cast<const int4*>(piece);
         }
       }
       if (low && high) side += YR * SW;
@@ -962,8 +887,8 @@ struct TileRows {
     if (threadIdx.x == 0) mbar_expect(&sm.bar, (unsigned)(Q * BOX * (int)sizeof(T)));
     const int i = (int)(threadIdx.x / 32) + NW * (int)(threadIdx.x % 32);
     if (i < Q)
-      tma_load5(sm.stage + i * IS, map, x0 - E, y0 - 1 - dir_y_rt(i),
-                source_plane(zp, dir_z_rt(i)) + (Shift ? kGhosts : 0), i, 0, &sm.bar);
+      tma_load4(sm.stage + i * IS, map, x0 - E, y0 - 1 - dir_y_rt(i),
+                source_plane(zp, dir_z_rt(i)) + (Shift ? kGhosts : 0), i, &sm.bar);
     side_pieces<true>(zp);
     cp_async_commit();
   }
@@ -984,15 +909,13 @@ struct TileRows {
   // is the site's (index s) own opposite one instead.
   template <int I>
   __device__ __forceinline__ float2 staged(int ly, int lx) const {
-    const T* q = sm.stage + (ly + 1) * SW + lx + E + (I * IS - dir_x(I));
-    return Pair<S>::cv(q[0], q[RH * SW], wgt(I));
+    return S::cv(sm.stage[(ly + 1) * SW + lx + E + (I * IS - dir_x(I))], wgt(I));
   }
   template <int I>
   __device__ __forceinline__ float2 pulled(int ly, int lx, bool sol_m, bool sol_p, Index s) const {
     constexpr int ez = dir_z(I);
     if (ez != 0 && (ez > 0 ? sol_m : sol_p)) {
-      const T* p = src + (long long)opp(I) * L.np + s;
-      return make_float2(S::ld(p, wgt(I)), S::ld(p + (long long)Q * L.np, wgt(I)));
+      return ld<S>(src + (long long)opp(I) * L.np + s, wgt(I));
     }
     return staged<I>(ly, lx);
   }
@@ -1140,13 +1063,11 @@ __device__ __forceinline__ void aa_slot(const PullIdx& P, int& idx, int& d) {
 template <class S, bool ODD>
 __device__ __forceinline__ void aa_load(const LatDev& L, const typename S::T* A, const PullIdx& P,
                                         float2 (&f)[Q]) {
-  const long long cstride = (long long)Q * L.np;
   Unroll<0, Q>::run([&](auto ic) {
     constexpr int I = decltype(ic)::value;
     int idx, d;
     aa_slot<I, ODD>(P, idx, d);
-    const typename S::T* p = A + (long long)d * L.np + idx;
-    f[I] = Pair<S>::cv(p[0], p[cstride], wgt(I));
+    f[I] = S::cv(A[(long long)d * L.np + idx], wgt(I));
   });
 }
 
@@ -1155,13 +1076,11 @@ __device__ __forceinline__ void aa_load(const LatDev& L, const typename S::T* A,
 template <class S, bool ODD>
 __device__ __forceinline__ void aa_load_cg(const LatDev& L, const typename S::T* A, const PullIdx& P,
                                            float2 (&f)[Q]) {
-  const long long cstride = (long long)Q * L.np;
   Unroll<0, Q>::run([&](auto ic) {
     constexpr int I = decltype(ic)::value;
     int idx, d;
     aa_slot<I, ODD>(P, idx, d);
-    const typename S::T* p = A + (long long)d * L.np + idx;
-    f[I] = make_float2(S::ldcg(p, wgt(I)), S::ldcg(p + cstride, wgt(I)));
+    f[I] = ldcg<S>(A + (long long)d * L.np + idx, wgt(I));
   });
 }
 
@@ -1169,13 +1088,11 @@ __device__ __forceinline__ void aa_load_cg(const LatDev& L, const typename S::T*
 template <class S, bool ODD>
 __device__ __forceinline__ void aa_store(const LatDev& L, typename S::T* A, const PullIdx& P,
                                          const float2 (&f)[Q]) {
-  const long long cstride = (long long)Q * L.np;
   Unroll<0, Q>::run([&](auto jc) {
     constexpr int J = decltype(jc)::value;
     int idx, d;
     aa_slot<opp(J), ODD>(P, idx, d);
-    typename S::T* p = A + (long long)d * L.np + idx;
-    Pair<S>::st(p, p + cstride, f[J], wgt(J));
+    put<S>(A + (long long)d * L.np + idx, f[J], wgt(J));
   });
 }
 

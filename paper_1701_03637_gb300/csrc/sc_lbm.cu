@@ -750,7 +750,6 @@ __global__ void k_load(const LatDev L, typename S::T* __restrict__ dst, long lon
     }
     // inverse of the pull: f_i(x) is read from x - e_i (wrapped), or from (x, opp(i))
     // when plane z - e_iz is solid.
-    const long long cstride = (long long)Q * L.np;
     Unroll<0, Q>::run([&](auto ic) {
       constexpr int I = decltype(ic)::value;
       const int zs = wrapi(z - dir_z(I), L.nz);
@@ -758,8 +757,7 @@ __global__ void k_load(const LatDev L, typename S::T* __restrict__ dst, long lon
       const int idx = sol ? x + L.nx * y + L.nxny * z
                           : wrapi(x - dir_x(I), L.nx) + L.nx * wrapi(y - dir_y(I), L.ny) + L.nxny * zs;
       const int d = sol ? opp(I) : I;
-      typename S::T* p = dst + (long long)d * L.np + idx;
-      Pair<S>::st(p, p + cstride, f[I], wgt(I));
+      put<S>(dst + (long long)d * L.np + idx, f[I], wgt(I));
     });
   }
 }
@@ -876,7 +874,7 @@ Layout make_layout(const sc_params* p) {
   l.tx = kTileX[l.tile];
   l.ty = kTileY[l.tile];
   l.aa = p->layout == SC_LAYOUT_AA;
-  l.rows = !l.aa && (p->staging == SC_STAGING_ROWS || (p->staging == SC_STAGING_AUTO && p->nx % (16 / es) == 0));
+  l.rows = !l.aa && (p->staging == SC_STAGING_ROWS || (p->staging == SC_STAGING_AUTO && p->nx % (8 / es) == 0));
   l.nsites = (long long)p->nx * p->ny * p->nz;
   l.np = round_up(l.nsites, 128 / es);  // each array starts 128-byte aligned
   l.stage_n = round_up(l.nsites, 64);
@@ -905,7 +903,7 @@ Layout make_layout(const sc_params* p) {
   if (l.planes > 0) {
     l.aa = false;
     l.shift = l.rows = true;
-    const size_t plane = (size_t)p->nx * p->ny * es;
+    const size_t plane = (size_t)p->nx * p->ny * 2 * es;
     l.off_pop[0] = kGhosts * plane;
     l.off_pop[1] = (kGhosts + l.planes) * plane;
     l.off_psi = off;
@@ -1046,8 +1044,8 @@ struct LaunchCfg {
 
 // Tensor map of a population buffer for the staged rows of a tile shape (a shifted lattice's
 // starts at the copied planes below plane 0 and covers those above too): dimensions
-// (x, y, z, direction, component), a box of one direction's TX + 2 E columns and TY + 2
-// rows of one plane, both components.
+// (x, y, z, direction) of pairs, a box of one direction's TX + 2 E columns and TY + 2
+// rows of one plane.
 using EncodeFn = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
                               const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
                               CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
@@ -1062,16 +1060,14 @@ int encode_map(const sc_lbm* h, const void* pop, int tile, CUtensorMap* m) {
       encode = (EncodeFn)fn;
   });
   if (!encode) return fail(SC_ECUDA, "the driver has no cuTensorMapEncodeTiled");
-  const cuuint64_t es = elem_size(h->p.storage);
-  const CUtensorMapDataType type = h->p.storage == SC_STORAGE_F32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32
-                                 : h->p.storage == SC_STORAGE_BF16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16
-                                                                   : CU_TENSOR_MAP_DATA_TYPE_FLOAT16;
+  const cuuint64_t ps = 2 * elem_size(h->p.storage);  // bytes of a pair
+  const CUtensorMapDataType type = ps == 8 ? CU_TENSOR_MAP_DATA_TYPE_UINT64 : CU_TENSOR_MAP_DATA_TYPE_UINT32;
   const cuuint64_t nx = h->p.nx, ny = h->p.ny, np = h->lay.np;
-  const cuuint64_t dims[5] = {nx, ny, (cuuint64_t)(h->p.nz + (h->lay.shift ? 2 * kGhosts : 0)), Q, 2};
-  const cuuint64_t strides[4] = {nx * es, nx * ny * es, np * es, Q * np * es};
-  const cuuint32_t box[5] = {(cuuint32_t)(kTileX[tile] + 2 * (16 / es)), (cuuint32_t)(kTileY[tile] + 2), 1, 1, 2};
-  const cuuint32_t unit[5] = {1, 1, 1, 1, 1};
-  const CUresult r = encode(m, type, 5, const_cast<void*>(pop), dims, strides, box, unit, CU_TENSOR_MAP_INTERLEAVE_NONE,
+  const cuuint64_t dims[4] = {nx, ny, (cuuint64_t)(h->p.nz + (h->lay.shift ? 2 * kGhosts : 0)), Q};
+  const cuuint64_t strides[3] = {nx * ps, nx * ny * ps, np * ps};
+  const cuuint32_t box[4] = {(cuuint32_t)(kTileX[tile] + 2 * (16 / ps)), (cuuint32_t)(kTileY[tile] + 2), 1, 1};
+  const cuuint32_t unit[4] = {1, 1, 1, 1};
+  const CUresult r = encode(m, type, 4, const_cast<void*>(pop), dims, strides, box, unit, CU_TENSOR_MAP_INTERLEAVE_NONE,
                             CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (r != CUDA_SUCCESS) return fail(SC_ECUDA, "cuTensorMapEncodeTiled failed: %d", (int)r);
@@ -2104,17 +2100,17 @@ int sc_slab_info(sc_lbm* h, int32_t* z0, int32_t* z1, int32_t* ghosts, size_t* f
   return SC_OK;
 }
 
-// The kSlabGhosts planes starting at local plane zl of the current buffer, as 2 * 19
-// arrays of kSlabGhosts * nx * ny elements each, to or from a packed device buffer.
+// The kSlabGhosts planes starting at local plane zl of the current buffer, as 19
+// arrays of kSlabGhosts * nx * ny pairs each, to or from a packed device buffer.
 static int slab_copy(sc_lbm* h, int zl, void* packed, bool to_packed) {
-  const size_t es = elem_size(h->p.storage);
-  const size_t run = (size_t)kSlabGhosts * h->p.nx * h->p.ny * es;  // contiguous in each array
-  char* planes = (char*)h->pop(h->cur) + (size_t)zl * h->p.nx * h->p.ny * es;
-  const size_t pitch = (size_t)h->lay.np * es;
+  const size_t ps = 2 * elem_size(h->p.storage);
+  const size_t run = (size_t)kSlabGhosts * h->p.nx * h->p.ny * ps;  // contiguous in each array
+  char* planes = (char*)h->pop(h->cur) + (size_t)zl * h->p.nx * h->p.ny * ps;
+  const size_t pitch = (size_t)h->lay.np * ps;
   if (to_packed)
-    CK(cudaMemcpy2DAsync(packed, run, planes, pitch, run, 2 * Q, cudaMemcpyDeviceToDevice, h->stream));
+    CK(cudaMemcpy2DAsync(packed, run, planes, pitch, run, Q, cudaMemcpyDeviceToDevice, h->stream));
   else
-    CK(cudaMemcpy2DAsync(planes, pitch, packed, run, run, 2 * Q, cudaMemcpyDeviceToDevice, h->stream));
+    CK(cudaMemcpy2DAsync(planes, pitch, packed, run, run, Q, cudaMemcpyDeviceToDevice, h->stream));
   return SC_OK;
 }
 

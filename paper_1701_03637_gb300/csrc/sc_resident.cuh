@@ -5,7 +5,7 @@
 // A lattice of a few thousand sites is bound by latency: a launch per step cost 10.5 us
 // (4x4x128, FP32, graphs of 64 launches), of which the arithmetic is under 1 us. Here CTA
 // r of a cluster of C holds sites [r ML, (r + 1) ML), one per thread, as two buffers
-// f[direction and component][site] in the storage type plus Psi; a step is
+// f[direction][site] of pairs in the storage type plus Psi; a step is
 //   pull the 19 directions of both components from the current buffer (the own CTA's or
 //   another's shared memory), densities, sink, Psi | cluster barrier | force from the
 //   neighbours' Psi, collision, store to the other buffer | cluster barrier.
@@ -33,19 +33,15 @@ __device__ __forceinline__ unsigned map_rank(unsigned addr, unsigned rank) {
 __device__ __forceinline__ void cluster_barrier() {
   asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;\n" ::: "memory");
 }
-__device__ __forceinline__ float ld_cluster(unsigned addr, float) {
-  float v;
-  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(addr) : "memory");
+__device__ __forceinline__ float2 ld_cluster(unsigned addr, float2) {
+  float2 v;
+  asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(addr) : "memory");
   return v;
 }
-__device__ __forceinline__ unsigned short ld_cluster16(unsigned addr) {
-  unsigned short v;
-  asm volatile("ld.shared::cluster.u16 %0, [%1];" : "=h"(v) : "r"(addr) : "memory");
+__device__ __forceinline__ uint32_t ld_cluster(unsigned addr, uint32_t) {
+  uint32_t v;
+  asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
   return v;
-}
-__device__ __forceinline__ __half ld_cluster(unsigned addr, __half) { return __ushort_as_half(ld_cluster16(addr)); }
-__device__ __forceinline__ __nv_bfloat16 ld_cluster(unsigned addr, __nv_bfloat16) {
-  return __ushort_as_bfloat16(ld_cluster16(addr));
 }
 
 // Bytes of shared memory for ML sites: the two buffers, then (Psi^r, Psi^b) of ML sites
@@ -61,7 +57,7 @@ __global__ void __launch_bounds__(kResidentThreads, 1)
   using T = typename S::T;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   T* f_sm = reinterpret_cast<T*>(smem_raw);
-  float2* psi_sm = reinterpret_cast<float2*>(smem_raw + resident_pop_bytes((int)sizeof(T), ML));
+  float2* psi_sm = reinterpret_cast<float2*>(smem_raw + resident_pop_bytes((int)sizeof(T) / 2, ML));
   const int n = L.nxny * L.nz, local = (int)threadIdx.x;
   const unsigned rank = cluster_rank();
   const int s = (int)rank * ML + local;
@@ -71,7 +67,7 @@ __global__ void __launch_bounds__(kResidentThreads, 1)
   const int cls = held ? site_class(L, x, y, z) : SOLID;
   const bool live = cls != SOLID;
 
-  unsigned fa[Q], pa[Q];  // source population (buffer 0, component r) and Psi of site x - e_I
+  unsigned fa[Q], pa[Q];  // source pair (buffer 0) and Psi of site x - e_I
   const unsigned f_base = smem_addr(f_sm), p_base = smem_addr(psi_sm);
   {
     const PullIdx P(L, x, y, z);
@@ -87,20 +83,20 @@ __global__ void __launch_bounds__(kResidentThreads, 1)
   }
   if (held) {
 #pragma unroll 1
-    for (int d = 0; d < 2 * Q; ++d) f_sm[d * ML + local] = pop[(long long)d * L.np + s];
+    for (int d = 0; d < Q; ++d) f_sm[d * ML + local] = pop[(long long)d * L.np + s];
   }
   if (threadIdx.x == 0) psi_sm[ML] = make_float2(0.f, 0.f);
-  const unsigned coff = (unsigned)(Q * ML * (int)sizeof(T));
+  const unsigned bytes = (unsigned)(Q * ML * (int)sizeof(T));
   double evap = 0.0;
   cluster_barrier();
 #pragma unroll 1
   for (int k = 0; k < K; ++k) {
-    const unsigned boff = (k & 1) ? 2u * coff : 0u;
+    const unsigned boff = (k & 1) ? bytes : 0u;
     float2 f[Q], rho = make_float2(0.f, 0.f), ps = rho;
     if (live) {
       Unroll<0, Q>::run([&](auto ic) {
         constexpr int I = decltype(ic)::value;
-        f[I] = Pair<S>::cv(ld_cluster(fa[I] + boff, T()), ld_cluster(fa[I] + boff + coff, T()), wgt(I));
+        f[I] = S::cv(ld_cluster(fa[I] + boff, T()), wgt(I));
       });
       rho = sum19(f);
       if (cls == SINK) {
@@ -119,27 +115,20 @@ __global__ void __launch_bounds__(kResidentThreads, 1)
         float2 a[3];
         force_sums_by_direction([&](auto ic) {
           constexpr int I = decltype(ic)::value;
-          float2 v;
-          asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(pa[I]) : "memory");
-          return v;
+          return ld_cluster(pa[I], float2());
         }, a);
         collide(L, f, rho, ps, a);
       }
-      T* to = f_sm + ((k & 1) ? 0 : 2 * Q * ML) + local;
+      T* to = f_sm + ((k & 1) ? 0 : Q * ML) + local;
 #pragma unroll
-      for (int i = 0; i < Q; ++i) {
-        T r, b;
-        Pair<S>::enc(f[i], wgt(i), r, b);
-        to[i * ML] = r;
-        to[(Q + i) * ML] = b;
-      }
+      for (int i = 0; i < Q; ++i) to[i * ML] = S::enc(f[i], wgt(i));
     }
     cluster_barrier();
   }
   if (held) {
-    const T* from = f_sm + ((K & 1) ? 2 * Q * ML : 0) + local;
+    const T* from = f_sm + ((K & 1) ? Q * ML : 0) + local;
 #pragma unroll 1
-    for (int d = 0; d < 2 * Q; ++d) pop[(long long)d * L.np + s] = from[d * ML];
+    for (int d = 0; d < Q; ++d) pop[(long long)d * L.np + s] = from[d * ML];
   }
   if (L.geometry != 0) {
     __shared__ double red[kResidentThreads / 32];

@@ -1,7 +1,7 @@
 // Shifted step: one population lattice advanced in its own storage by the two-lattice step's
 // staged-rows march. Included by sc_lbm.cu, whose handle and helpers it shares.
 //
-// The 38 arrays have nz + s + 4 planes. In state 0 the lattice lies in planes [2, nz + 2), in
+// The 19 arrays of pairs have nz + s + 4 planes. In state 0 the lattice lies in planes [2, nz + 2), in
 // state 1 in planes [s + 2, nz + s + 2); a step reads one and writes the other, so plane z is
 // written s planes away from where it is read, over old plane z - s (state 1 -> 0, marching up)
 // or z + s (0 -> 1, marching down). The work is cut into chunks of at most s - 2 planes, claimed
@@ -16,7 +16,7 @@
 // Why: in place, the force needs Psi of a neighbour before that neighbour is overwritten, so
 // the AA steps read every population twice, and on a 512^2 plane (40 MB per plane, three in
 // use) the second read misses the L2. Here it is read once, plus the halo planes of the chunks:
-// 512^3 FP32, 20 steps 234 (persistent) -> 196 ms, 9.8 ms per step against a floor of 6.0; what
+// 512^3 FP32, 20 steps 234 (persistent) -> 184 ms, 9.2 ms per step against a floor of 6.0; what
 // is left beyond the two-lattice step's 7.3 ms is the chunks of 19 planes (two planes staged
 // for nothing per chunk) and a register spill in the march.
 
@@ -30,11 +30,11 @@ constexpr int kShiftMinChunk = 6;  // planes; shorter chunks stage too many halo
 constexpr int kShiftMinCols = 384;
 constexpr int kShiftReach = 2;     // tile columns on each side whose items may read a tile's sites
 
-// Planes that the lattice moves by: the Psi array's memory as extra planes of the 38 arrays,
+// Planes that the lattice moves by: the Psi array's memory as extra planes of the 19 arrays,
 // less the copied ones. 0 where the shifted step does not apply.
 int shift_planes(const sc_params* p, long long es, long long bytes, long long* np) {
   if (p->layout != SC_LAYOUT_AA || p->staging != SC_STAGING_AUTO || p->tile != 0 || p->zchunk != 0 || p->nx < 64 ||
-      p->nx % (16 / es) != 0)
+      p->nx % (8 / es) != 0)
     return 0;
   const long long cols = (long long)((p->nx + 63) / 64) * ((p->ny + 3) / 4);
   if (cols > 2 * kMaxCtas || cols < kShiftMinCols) return 0;
@@ -63,12 +63,12 @@ struct ShiftArgs {
   long long limit_ns;   // of a wait
 };
 
-// Copies `n16` 16-byte pieces (two planes) of each of the 2 Q arrays and clears the column counters.
+// Copies `n16` 16-byte pieces (two planes) of each of the Q arrays and clears the column counters.
 __global__ void __launch_bounds__(256) k_shift_begin(const int4* __restrict__ from, int4* __restrict__ to,
                                                      long long stride16, int n16, unsigned* __restrict__ done, int cols) {
   const long long t = blockIdx.x * 256LL + threadIdx.x, step = gridDim.x * 256LL;
   for (long long k = t; k < cols; k += step) done[k] = 0u;
-  for (long long k = t; k < 2LL * Q * n16; k += step) {
+  for (long long k = t; k < (long long)Q * n16; k += step) {
     const long long a = k / n16, o = a * stride16 + (k - a * n16);
     to[o] = from[o];
   }
@@ -167,7 +167,7 @@ int plan_shift(sc_lbm* h) {
   h->wait_limit_ns = 2000000000LL;
   h->withhold = -1;
   for (int k = 0; k < 2; ++k) {
-    const int rc = encode_map(h, (char*)h->pop(k) - (size_t)kGhosts * h->L.nxny * elem_size(h->p.storage), l.tile,
+    const int rc = encode_map(h, (char*)h->pop(k) - (size_t)kGhosts * h->L.nxny * 2 * elem_size(h->p.storage), l.tile,
                               &h->maps[k]);
     if (rc) return rc;
   }
@@ -186,7 +186,7 @@ cudaError_t launch_shift(sc_lbm* h, cudaStream_t st) {
   T* to = const_cast<T*>(down ? src - kGhosts * plane : src + nz * plane);
   const int n16 = (int)(kGhosts * plane / E);
   unsigned* done = (unsigned*)h->flags();
-  k_shift_begin<<<grid_for(2LL * Q * n16, 1024), 256, 0, st>>>((const int4*)from, (int4*)to, h->L.np / E, n16, done, l.cols);
+  k_shift_begin<<<grid_for((long long)Q * n16, 1024), 256, 0, st>>>((const int4*)from, (int4*)to, h->L.np / E, n16, done, l.cols);
   const ShiftArgs a{l.cols_x, l.cols / l.cols_x, h->nitems, (int)l.nslots, down, h->next(), done, h->h_err, h->wait_limit_ns};
   k_shift<64, 4, S><<<h->grid, 256, shift_smem<S>(h->L), st>>>(h->L, src, (T*)h->pop(1 - h->cur), h->evap(), a,
                                                                h->maps[h->cur]);

@@ -1040,6 +1040,7 @@ struct sc_lbm {
   int zmax;  // planes of the longest work item
   int nitems;  // work items of a step (two lattices)
   int rcta, rsites;  // resident step: CTAs of its cluster (0: not used) and sites of each
+  bool rplanes;      // whole planes per CTA, with threads for the plane on each side
   cudaGraphExec_t graph;
   int graph_len;
   int graph_cur;

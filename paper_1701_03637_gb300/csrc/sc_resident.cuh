@@ -9,6 +9,10 @@
 //   pull the 19 directions of both components from the current buffer (the own CTA's or
 //   another's shared memory), densities, sink, Psi | cluster barrier | force from the
 //   neighbours' Psi, collision, store to the other buffer | cluster barrier.
+// Where a CTA holds whole planes and has threads to spare for the plane on each side (PLANES),
+// these form that plane's Psi from its populations (the owner's arithmetic, so its bits): Psi
+// is then shared within the CTA and the first cluster barrier is a CTA barrier: 100 film steps
+// with diagnostics and read-out 168 -> 155 us.
 // The addresses of the 19 sources are the same in every step and stay in registers (a
 // population next to a wall is the site's own opposite one, and a solid neighbour's Psi a
 // cell that holds 0), so a step has no index arithmetic. Values are rounded to the
@@ -45,13 +49,15 @@ __device__ __forceinline__ uint32_t ld_cluster(unsigned addr, uint32_t) {
 }
 
 // Bytes of shared memory for ML sites: the two buffers, then (Psi^r, Psi^b) of ML sites
-// and the cell that holds 0.
+// and of `extra`: the planes on each side, or the cell that holds 0.
 __host__ __device__ constexpr size_t resident_pop_bytes(int es, int ML) {
   return ((size_t)2 * 2 * Q * ML * es + 15) / 16 * 16;
 }
-constexpr size_t resident_smem(int es, int ML) { return resident_pop_bytes(es, ML) + sizeof(float2) * ((size_t)ML + 1); }
+constexpr size_t resident_smem(int es, int ML, int extra) {
+  return resident_pop_bytes(es, ML) + sizeof(float2) * ((size_t)ML + extra);
+}
 
-template <class S>
+template <class S, bool PLANES>
 __global__ void __launch_bounds__(kResidentThreads, 1)
     k_resident(const LatDev L, typename S::T* __restrict__ pop, double* __restrict__ evap_cum, int K, int ML) {
   using T = typename S::T;
@@ -64,7 +70,24 @@ __global__ void __launch_bounds__(kResidentThreads, 1)
   const bool held = local < ML && s < n;
   int x = 0, y = 0, z = 0;
   if (held) site_of(L, s, x, y, z);
-  const int cls = held ? site_class(L, x, y, z) : SOLID;
+  // Psi cell: own sites in order, with PLANES after the plane below, and the one above next
+  const int mine = min(ML, n - (int)rank * ML);  // the CTA's sites (whole planes with PLANES)
+  int cell = PLANES ? local + L.nxny : local;
+  bool halo = false;
+  if (PLANES && local >= ML && mine > 0) {
+    const int q = local - ML;  // a site of the plane below or above
+    halo = q < 2 * L.nxny;
+    if (halo) {
+      const bool above = q >= L.nxny;
+      const int in_plane = above ? q - L.nxny : q;
+      const int zb = ((int)rank * ML) / L.nxny, ze = zb + mine / L.nxny;
+      x = in_plane % L.nx;
+      y = in_plane / L.nx;
+      z = above ? (ze == L.nz ? 0 : ze) : (zb == 0 ? L.nz - 1 : zb - 1);
+      cell = in_plane + (above ? L.nxny + mine : 0);
+    }
+  }
+  const int cls = held || halo ? site_class(L, x, y, z) : SOLID;
   const bool live = cls != SOLID;
 
   unsigned fa[Q], pa[Q];  // source pair (buffer 0) and Psi of site x - e_I
@@ -77,6 +100,10 @@ __global__ void __launch_bounds__(kResidentThreads, 1)
       P.template at<I>(idx, d);
       const int owner = idx / ML, loc = idx - owner * ML;
       fa[I] = map_rank(f_base + (unsigned)((d * ML + loc) * (int)sizeof(T)), (unsigned)owner);
+      if constexpr (PLANES) {  // site x - e_I within the CTA; 0 is stored at solid sites
+        const int xs = P.xs[1 + dir_x(I)], ys = P.ys[1 + dir_y(I)];
+        pa[I] = p_base + (unsigned)((held ? cell - y * L.nx - x - dir_z(I) * L.nxny + ys + xs : 0) * (int)sizeof(float2));
+      } else
       pa[I] = d == I ? map_rank(p_base + (unsigned)(loc * (int)sizeof(float2)), (unsigned)owner)
                      : p_base + (unsigned)(ML * (int)sizeof(float2));
     });
@@ -85,7 +112,7 @@ __global__ void __launch_bounds__(kResidentThreads, 1)
 #pragma unroll 1
     for (int d = 0; d < Q; ++d) f_sm[d * ML + local] = pop[(long long)d * L.np + s];
   }
-  if (threadIdx.x == 0) psi_sm[ML] = make_float2(0.f, 0.f);
+  if (!PLANES && threadIdx.x == 0) psi_sm[ML] = make_float2(0.f, 0.f);
   const unsigned bytes = (unsigned)(Q * ML * (int)sizeof(T));
   double evap = 0.0;
   cluster_barrier();
@@ -100,14 +127,15 @@ __global__ void __launch_bounds__(kResidentThreads, 1)
       });
       rho = sum19(f);
       if (cls == SINK) {
-        evap += (double)sink_excess(L, f);
+        if (held) evap += (double)sink_excess(L, f);
         sink_densities(L, rho);
       }
       ps = psi_of(rho);
     }
-    if (held) psi_sm[local] = ps;
-    cluster_barrier();
-    if (live) {
+    if (held || halo) psi_sm[cell] = ps;
+    if constexpr (PLANES) __syncthreads();
+    else cluster_barrier();
+    if (live && held) {
       if (cls == SINK) {
 #pragma unroll
         for (int i = 0; i < Q; ++i) f[i] = rest_pop(i, rho);
@@ -145,20 +173,25 @@ __global__ void __launch_bounds__(kResidentThreads, 1)
   }
 }
 
-void* resident_fn(int storage) {
+template <bool PLANES>
+void* resident_fn_of(int storage) {
   switch (storage) {
-    case SC_STORAGE_F16: return (void*)k_resident<StF16>;
-    case SC_STORAGE_F16_SCALED: return (void*)k_resident<StF16S>;
-    case SC_STORAGE_BF16: return (void*)k_resident<StBF16>;
-    default: return (void*)k_resident<StF32>;
+    case SC_STORAGE_F16: return (void*)k_resident<StF16, PLANES>;
+    case SC_STORAGE_F16_SCALED: return (void*)k_resident<StF16S, PLANES>;
+    case SC_STORAGE_BF16: return (void*)k_resident<StBF16, PLANES>;
+    default: return (void*)k_resident<StF32, PLANES>;
   }
+}
+void* resident_fn(const sc_lbm* h) {
+  return h->rplanes ? resident_fn_of<true>(h->p.storage) : resident_fn_of<false>(h->p.storage);
 }
 
 void resident_config(const sc_lbm* h, cudaLaunchConfig_t* cfg, cudaLaunchAttribute* at, cudaStream_t st) {
   *cfg = cudaLaunchConfig_t{};
   cfg->gridDim = dim3((unsigned)h->rcta);
-  cfg->blockDim = dim3((unsigned)(round_up(h->rsites, 32)));
-  cfg->dynamicSmemBytes = resident_smem((int)elem_size(h->p.storage), h->rsites);
+  const int extra = 2 * h->L.nxny;
+  cfg->blockDim = dim3((unsigned)round_up(h->rsites + (h->rplanes ? extra : 0), 32));
+  cfg->dynamicSmemBytes = resident_smem((int)elem_size(h->p.storage), h->rsites, h->rplanes ? extra : 1);
   cfg->stream = st;
   at->id = cudaLaunchAttributeClusterDimension;
   at->val.clusterDim.x = (unsigned)h->rcta;
@@ -180,15 +213,16 @@ void plan_resident(sc_lbm* h) {
   int c = 1;
   while (c < kResidentCluster && n > 128LL * c) c *= 2;
   for (; c >= 1; c /= 2) {
-    const long long ml = (n + c - 1) / c;
+    const long long ml = (n + c - 1) / c, plane = h->L.nxny, whole = (ml + plane - 1) / plane * plane;
     if (ml > kResidentThreads || c > h->lay.nslots) continue;
     h->rcta = c;
-    h->rsites = (int)ml;
+    h->rplanes = whole + 2 * plane <= kResidentThreads;
+    h->rsites = (int)(h->rplanes ? whole : ml);
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute at;
     resident_config(h, &cfg, &at, h->stream);
-    void* fn = resident_fn(p.storage);
-    const int most = (int)resident_smem((int)elem_size(p.storage), kResidentThreads);
+    void* fn = resident_fn(h);
+    const int most = (int)resident_smem((int)elem_size(p.storage), kResidentThreads, 1);
     int clusters = 0;
     if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, most) == cudaSuccess &&
         cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
@@ -210,7 +244,7 @@ int launch_resident(sc_lbm* h, int64_t nsteps) {
     double* evap = h->evap();
     int K = (int)std::min<int64_t>(left, kResidentMaxSteps), ML = h->rsites;
     void* args[] = {&L, &pop, &evap, &K, &ML};
-    const cudaError_t e = cudaLaunchKernelExC(&cfg, resident_fn(h->p.storage), args);
+    const cudaError_t e = cudaLaunchKernelExC(&cfg, resident_fn(h), args);
     if (e != cudaSuccess) return fail(SC_ECUDA, "resident step launch failed: %s", cudaGetErrorString(e));
   }
   return SC_OK;

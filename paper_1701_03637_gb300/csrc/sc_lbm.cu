@@ -1816,8 +1816,25 @@ int sc_lbm_step(sc_lbm* h, int64_t nsteps) {
 
 int sc_lbm_read_fields_device(sc_lbm* h, float* rr, float* rb) {
   if (!h || !rr || !rb) return fail(SC_EINVAL, "NULL argument");
-  // the kernel writes the caller's arrays (rho^b at their distance from rho^r)
-  return canonical(h, 0, h->lay.nsites, rr, rb - rr, nullptr, 0);
+  const long long n = h->lay.nsites;
+  // the kernel writes the caller's arrays (rho^b at their distance from rho^r) where it can
+  // reach them; overlapping, unaligned, host and other devices' memory takes a copy
+  int dev = 0;
+  CK(cudaGetDevice(&dev));
+  const intptr_t apart = (intptr_t)rb - (intptr_t)rr, bytes = (intptr_t)(sizeof(float) * n);
+  bool direct = (((uintptr_t)rr | (uintptr_t)rb) & 3) == 0 && (apart >= bytes || apart <= -bytes);
+  for (const float* p : {rr, rb}) {
+    cudaPointerAttributes at{};
+    if (!direct) break;
+    if (cudaPointerGetAttributes(&at, p) != cudaSuccess) cudaGetLastError();
+    direct = at.type == cudaMemoryTypeDevice && at.device == dev;
+  }
+  if (direct) return canonical(h, 0, n, rr, apart / (intptr_t)sizeof(float), nullptr, 0);
+  const int rc = canonical(h, 0, n, h->stage(), h->lay.stage_n, nullptr, 0);
+  if (rc) return rc;
+  CK(cudaMemcpyAsync(rr, h->stage(), sizeof(float) * n, cudaMemcpyDeviceToDevice, h->stream));
+  CK(cudaMemcpyAsync(rb, h->stage() + h->lay.stage_n, sizeof(float) * n, cudaMemcpyDeviceToDevice, h->stream));
+  return SC_OK;
 }
 
 int sc_lbm_read_fields(sc_lbm* h, float* rr, float* rb) {

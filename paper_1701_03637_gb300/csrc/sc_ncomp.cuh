@@ -6,7 +6,8 @@
 //
 // Periodic lattice with an optional solid slab (halfway bounce-back, Psi = 0 at
 // solid sites); no evaporation sink (the paper states it for two components).
-// Two population lattices of FP32 arrays f[c][i][s]; each step is one launch of
+// Two population lattices of FP32 arrays f[c][i][s]; small lattices take two launches per step
+// (k_n_psi, k_n_collide), others one of
 // k_n_step: a CTA of 32 x 8 threads owns a tile column and a chunk of its planes and
 // marches them, forming Psi^c of plane p + 1 over the tile and a one-site halo from
 // the pulled populations into a shared ring of 4 planes, then pulling plane p again
@@ -72,13 +73,12 @@ __device__ __forceinline__ void n_psi_plane(const NDev& D, const float* __restri
   }
 }
 
-// Stream, force, common velocity and shifted relaxation of site (x, y, p) (tile cell
-// (tx, ty)), Psi from the ring; stores f*.
-template <int NC>
+// Stream, force, common velocity and shifted relaxation of the site of P; psi(c, I) yields
+// Psi^c of the site x - e_I. Stores f*.
+template <int NC, class PsiFrom>
 __device__ __forceinline__ void n_collide_site(const NDev& D, const float* __restrict__ src, float* __restrict__ dst,
-                                               const NRing<NC>& r, int p, int x, int y, int tx, int ty) {
+                                               const PullIdx& P, PsiFrom psi) {
   const LatDev& L = D.L;
-  const PullIdx P(L, x, y, p);
   const int s = P.s;
   float f[NC][Q], rho[NC], m[NC][3];
 #pragma unroll
@@ -101,13 +101,10 @@ __device__ __forceinline__ void n_collide_site(const NDev& D, const float* __res
     for (int c = NC - 2; c >= 0; --c) num = __fmaf_rn(m[c][d], D.om[c], num);
     up[d] = __fmul_rn(num, inv);
   }
-  // a^c = sum_i w_i Psi^c(x + e_i) e_i from the ring (planes p - 1, p, p + 1)
+  // a^c = sum_i w_i Psi^c(x + e_i) e_i
   float a[NC][3];
 #pragma unroll
-  for (int c = 0; c < NC; ++c) {
-    auto psi1 = [&](int sl, int yy, int xx) { return r.v[sl][c][yy + 1][xx + 1]; };
-    force_sums(psi1, (p - 1) & 3, p & 3, (p + 1) & 3, ty, tx, a[c]);
-  }
+  for (int c = 0; c < NC; ++c) force_sums_by_direction([&](auto ic) { return psi(c, ic); }, a[c]);
 #pragma unroll
   for (int c = 0; c < NC; ++c) {
     // A^c = sum_cbar g^{c cbar} a^cbar: the other components first (the first as a
@@ -125,7 +122,7 @@ __device__ __forceinline__ void n_collide_site(const NDev& D, const float* __res
       }
       A[d] = __fmaf_rn(D.g[c][c], a[c][d], acc);
     }
-    relax_core(D.om[c], D.tau[c], f[c], rho[c], r.v[p & 3][c][ty + 1][tx + 1], 1.0f, A, up);
+    relax_core(D.om[c], D.tau[c], f[c], rho[c], psi(c, std::integral_constant<int, 0>()), 1.0f, A, up);
 #pragma unroll
     for (int i = 0; i < Q; ++i) dst[((long long)c * Q + i) * L.np + s] = f[c][i];
   }
@@ -151,8 +148,52 @@ __global__ void __launch_bounds__(kNT) k_n_step(const NDev D, const float* __res
   for (int p = zb; p < ze; ++p) {
     n_psi_plane<NC>(D, src, r, p + 1, x0, y0);
     __syncthreads();
-    if (active && !solid_z(L, p)) n_collide_site<NC>(D, src, dst, r, p, x, y, tx, ty);
+    if (active && !solid_z(L, p))
+      n_collide_site<NC>(D, src, dst, PullIdx(L, x, y, p), [&](int c, auto ic) {
+        constexpr int I = decltype(ic)::value;
+        return r.v[(p - dir_z(I)) & 3][c][ty - dir_y(I) + 1][tx - dir_x(I) + 1];
+      });
   }
+}
+
+// The same step in two launches, a site per thread: Psi of every component into an array, then
+// the rest with Psi from there. No halo is formed twice and no CTA waits for another's plane,
+// but every population is read twice: for lattices whose two buffers stay in the L2. Bound by
+// the latency and the issue of its loads. Per step, marched against in two launches: 64^3 of 2
+// components 30.8 / 22.6 us, of 3 39.0 / 34.8; 48^3 of 3 22.6 / 20.5; beyond the L2 80^3 of 3
+// 75.8 / 81.9. With 4 components the marched step, which shares its index arithmetic among
+// them, stays ahead (32^3 12.3 / 14.2, 64^3 53.3 / 55.3).
+constexpr int kNSiteY = 4;  // rows of 32 sites per CTA
+constexpr size_t kNSitesBytes = 126000000;  // the L2
+template <int NC>
+__global__ void __launch_bounds__(32 * kNSiteY) k_n_psi(const NDev D, const float* __restrict__ src, float* __restrict__ psi) {
+  const LatDev& L = D.L;
+  const int x = blockIdx.x * 32 + threadIdx.x, y = blockIdx.y * kNSiteY + threadIdx.y, z = blockIdx.z;
+  if (x >= L.nx || y >= L.ny) return;
+  const PullIdx P(L, x, y, z);
+  const bool solid = solid_z(L, z);
+#pragma unroll
+  for (int c = 0; c < NC; ++c) {
+    float v = 0.f;
+    if (!solid) {
+      float f[Q];
+      pull_comp(L, src + (long long)c * Q * L.np, P, f);
+      v = psi_of(sum19(f));
+    }
+    psi[(long long)c * L.np + P.s] = v;
+  }
+}
+template <int NC>
+__global__ void __launch_bounds__(32 * kNSiteY) k_n_collide(const NDev D, const float* __restrict__ src,
+                                                            float* __restrict__ dst, const float* __restrict__ psi) {
+  const LatDev& L = D.L;
+  const int x = blockIdx.x * 32 + threadIdx.x, y = blockIdx.y * kNSiteY + threadIdx.y, z = blockIdx.z;
+  if (x >= L.nx || y >= L.ny || solid_z(L, z)) return;
+  const PullIdx P(L, x, y, z);
+  n_collide_site<NC>(D, src, dst, P, [&](int c, auto ic) {
+    constexpr int I = decltype(ic)::value;
+    return __ldg(psi + (long long)c * L.np + (P.xs[1 + dir_x(I)] + P.ys[1 + dir_y(I)] + P.zs[1 + dir_z(I)]));
+  });
 }
 
 // Canonical populations (pull) of every component into out[c][i][s] (dense, N sites).
@@ -245,6 +286,21 @@ cudaError_t n_step_launch(const NDev& D, const float* src, float* dst, int cols_
   return cudaGetLastError();
 }
 
+template <int NC>
+cudaError_t n_sites_launch(const NDev& D, const float* src, float* dst, float* psi, cudaStream_t st) {
+  const dim3 grid((D.L.nx + 31) / 32, (D.L.ny + kNSiteY - 1) / kNSiteY, D.L.nz), block(32, kNSiteY);
+  k_n_psi<NC><<<grid, block, 0, st>>>(D, src, psi);
+  k_n_collide<NC><<<grid, block, 0, st>>>(D, src, dst, psi);
+  return cudaGetLastError();
+}
+cudaError_t n_sites_dispatch(int nc, const NDev& D, const float* src, float* dst, float* psi, cudaStream_t st) {
+  switch (nc) {
+    case 2: return n_sites_launch<2>(D, src, dst, psi, st);
+    case 3: return n_sites_launch<3>(D, src, dst, psi, st);
+    default: return n_sites_launch<4>(D, src, dst, psi, st);
+  }
+}
+
 cudaError_t n_step_dispatch(int nc, const NDev& D, const float* src, float* dst, int cols_x, int cols, int nch,
                             cudaStream_t st) {
   switch (nc) {
@@ -273,7 +329,8 @@ struct sc_ncomp {
   size_t pop_bytes, off_pop[2], off_psi, total;
   int cur;
   int grid;                  // CTAs of the site-parallel kernels
-  int cols_x, cols, nch;     // the step's tile columns and plane chunks (cols * nch CTAs)
+  bool sites;                // the two-launch step
+  int cols_x, cols, nch;     // the marching step's tile columns and plane chunks (cols * nch CTAs)
   int64_t step;
   float* pop(int k) const { return (float*)(base + off_pop[k]); }
   float* psi() const { return (float*)(base + off_psi); }
@@ -313,6 +370,7 @@ int sc_ncomp_create(const sc_nparams* p, void* stream, sc_ncomp** out) {
   h->off_pop[1] = h->pop_bytes;
   h->off_psi = 2 * h->pop_bytes;
   h->total = h->off_psi + align256((size_t)p->ncomp * np * sizeof(float));
+  h->sites = p->ncomp <= 3 && 2 * h->pop_bytes <= kNSitesBytes && p->nz <= 65535 && p->ny <= 65535 * kNSiteY;
   h->stream = (cudaStream_t)stream;
   h->grid = (int)grid_for(l.nsites, 256);
   // plane chunks: the fewest waves of resident CTAs times the planes (with the two
@@ -403,7 +461,10 @@ int sc_ncomp_step(sc_ncomp* h, int64_t nsteps) {
   if (nsteps < 0) return fail(SC_EINVAL, "nsteps must be >= 0");
   for (int64_t k = 0; k < nsteps; ++k) {
     const int src = h->cur, dst = 1 - h->cur;
-    CK(n_step_dispatch(h->p.ncomp, h->D, h->pop(src), h->pop(dst), h->cols_x, h->cols, h->nch, h->stream));
+    if (h->sites)
+      CK(n_sites_dispatch(h->p.ncomp, h->D, h->pop(src), h->pop(dst), h->psi(), h->stream));
+    else
+      CK(n_step_dispatch(h->p.ncomp, h->D, h->pop(src), h->pop(dst), h->cols_x, h->cols, h->nch, h->stream));
     h->cur = dst;
   }
   h->step += nsteps;

@@ -97,9 +97,9 @@ extern "C" {
                                    Psi of every site into an FP32 (Psi^r, Psi^b) array, 8 bytes
                                    per site, then stream + sink + force + collision in place;
                                    472 bytes). With SC_STAGING_AUTO, tall lattices of large
-                                   planes (nx a multiple of 2 for FP32, of 4 for FP16/BF16, 384
+                                   planes (nx a multiple of 2 for FP32, of 4 for FP16/BF16, 576
                                    tiles of 64 x 4 sites per plane or more, and enough planes
-                                   that the Psi array's memory holds at least 12 of them) take
+                                   that the Psi array's memory holds at least 21 of them) take
                                    neither form: the lattice lies where the two-lattice step
                                    would keep it and is moved by some planes, alternately down
                                    and up, through storage that has the Psi array's memory as

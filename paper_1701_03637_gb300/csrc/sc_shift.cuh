@@ -22,12 +22,14 @@
 
 namespace {
 
-constexpr int kShiftMinChunk = 6;  // planes; shorter chunks stage too many halo planes
-// Tile columns: one per resident CTA (2 on each of 152 SMs) and a few rows of tiles more, so that
-// the chunk before is finished around an item's column when the item is claimed. With fewer the
-// items of two chunks wait for one another (FP32 256^3, 256 columns: 2.45 against 1.42 ms
-// for the two-pass step).
-constexpr int kShiftMinCols = 384;
+// Longest chunk: shorter ones read too many halo planes ((c + 4) / c; FP32 320^3, 10 planes: 3.36
+// against 2.85 ms for the two-pass step, 384^3, 12: 4.54 against 4.33; 448^3, 16: 6.2 against 7.6).
+constexpr int kShiftMinChunk = 15;
+// Tile columns: about two rounds of the resident CTAs (2 on each of 152 SMs), so that the chunk
+// before is finished around an item's column when the item is claimed. With fewer the items
+// wait for one another (FP16 320^3, 400 columns: 2.31 against 2.31 ms for the two-pass step;
+// 384^3, 576: 3.16 against 3.41; 512 x 512 x 256, 1024: 3.35 against 4.03).
+constexpr int kShiftMinCols = 576;
 constexpr int kShiftReach = 2;     // tile columns on each side whose items may read a tile's sites
 
 // Planes that the lattice moves by: the Psi array's memory as extra planes of the 19 arrays,

@@ -892,6 +892,27 @@ int auto_tile(const sc_params* p) {
 
 int shift_planes(const sc_params* p, long long es, long long bytes, long long* np);
 
+// Whether the automatic two-lattice step stages rows. A plane's rows are waited for, its
+// wrapped pieces moved from the side buffer and only then is it read out: a fixed cost per
+// plane, which shows where a tile is one warp (narrow lattices), where the tiles are few and
+// where the state stays in the L2. Per-thread pulls have no such step but issue a copy per
+// population.
+// us per step, rows / pulls (planar sink): FP32 10x10x256 18.1 / 11.0, 24x24x128 17.1 / 11.3,
+// 64^3 23.9 / 20.6, 64x64x128 36.9 / 36.4, 96^3 59.9 / 60.4, 128^3 132.8 / 138.3, 224^3 626 /
+// 683, 512x512x64 900 / 1007; with few rows or columns of tiles 1024x4x512 157 / 125, 512x8x512
+// 133 / 123, 1024x16x128 136 / 140, 36x200x256 174 / 154, 34x512x256 394 / 416. FP16 64^3 22.6 /
+// 19.6, 128^3 124.6 / 119.2, 256^3 782 / 759, 288^3 1076 / 1106, 512^3 5731 / 5826, 64x1024x512
+// 1488 / 1457, 384^3 with the spherical sink 2862 / 2776. So: FP32 where both buffers exceed
+// twice the L2 (from 4M sites under 64 columns), 16-bit types beyond 2^24 sites of 128 columns
+// or more without the spherical sink.
+constexpr long long kL2Bytes = 126000000;
+bool rows_pay(const sc_params* p, long long es) {
+  const long long n = (long long)p->nx * p->ny * p->nz;
+  if (p->nx % (8 / es) != 0 || p->nx < 32 || p->ny < 16) return false;
+  if (es == 2) return p->nx >= 128 && n > (1LL << 24) && p->geometry != SC_GEOM_SPHERE_SINK;
+  return p->nx < 64 ? n >= (1LL << 22) : 4 * Q * es * n > 2 * kL2Bytes;
+}
+
 Layout make_layout(const sc_params* p) {
   Layout l{};
   const long long es = (long long)elem_size(p->storage);
@@ -899,7 +920,7 @@ Layout make_layout(const sc_params* p) {
   l.tx = kTileX[l.tile];
   l.ty = kTileY[l.tile];
   l.aa = p->layout == SC_LAYOUT_AA;
-  l.rows = !l.aa && (p->staging == SC_STAGING_ROWS || (p->staging == SC_STAGING_AUTO && p->nx % (8 / es) == 0));
+  l.rows = !l.aa && (p->staging == SC_STAGING_ROWS || (p->staging == SC_STAGING_AUTO && rows_pay(p, es)));
   l.nsites = (long long)p->nx * p->ny * p->nz;
   l.np = round_up(l.nsites, 128 / es);  // each array starts 128-byte aligned
   l.stage_n = round_up(l.nsites, 64);

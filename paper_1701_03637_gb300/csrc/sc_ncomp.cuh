@@ -164,7 +164,7 @@ __global__ void __launch_bounds__(kNT) k_n_step(const NDev D, const float* __res
 // 75.8 / 81.9. With 4 components the marched step, which shares its index arithmetic among
 // them, stays ahead (32^3 12.3 / 14.2, 64^3 53.3 / 55.3).
 constexpr int kNSiteY = 4;  // rows of 32 sites per CTA
-constexpr size_t kNSitesBytes = 126000000;  // the L2
+constexpr size_t kNSitesBytes = kL2Bytes;
 template <int NC>
 __global__ void __launch_bounds__(32 * kNSiteY) k_n_psi(const NDev D, const float* __restrict__ src, float* __restrict__ psi) {
   const LatDev& L = D.L;

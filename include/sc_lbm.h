@@ -265,13 +265,14 @@ int sc_lbm_launch_count(sc_lbm* h, int64_t nsteps, int64_t* launches);
 /* Name of the kernel (or kernels) that carries the step in the current configuration,
    a static string ("" for a NULL handle). */
 const char* sc_lbm_kernel_name(sc_lbm* h);
-/* Time limit of each progress wait of the persistent in-place step (default 2 s), and a
-   test hook: CTA withhold_cta (-1: none) never reports its progress, so its neighbours'
-   waits run out after limit_ns. A wait that runs out ends the launch early; the state
-   is then undefined, sc_lbm_sync returns SC_ETIMEOUT and diagnostics report status
-   SC_ETIMEOUT until a state is loaded (sc_lbm_init, _init_fields, _write_populations).
-   Nothing waits without a limit, so the device stays usable. No counterpart in the
-   paper. */
+/* Time limit of each progress wait of the in-place steps that have them, the persistent and
+   the shifted one (default 2 s; SC_LAYOUT_AA), from the next step on, and a test hook: CTA
+   withhold_cta (-1: none; below the CTA count of sc_lbm_launch_info) never reports its
+   progress, so that its neighbours' waits run out after limit_ns. A wait that runs out ends
+   the step early; the state is then undefined, sc_lbm_sync returns SC_ETIMEOUT and
+   diagnostics report status SC_ETIMEOUT until a state is loaded (sc_lbm_init, _init_fields,
+   _write_populations). Nothing waits without a limit, so the device stays usable. Steps
+   without progress waits ignore both. No counterpart in the paper. */
 int sc_lbm_set_wait(sc_lbm* h, int64_t limit_ns, int32_t withhold_cta);
 /* Bands of the persistent in-place step. That step marches the lattice in `bands`
    bands of equal width along x, one after another within every step; each band is

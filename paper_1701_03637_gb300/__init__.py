@@ -262,8 +262,8 @@ class Lattice:
         return int(b.value)
 
     def set_wait(self, limit_ns: int, withhold_cta: int = -1) -> None:
-        """Time limit of the persistent in-place step's progress waits; withhold_cta >= 0
-        makes that CTA withhold its progress reports (a test of the failure path)."""
+        """Time limit of the progress waits of the persistent and the shifted in-place step;
+        withhold_cta >= 0 makes that CTA withhold its progress reports (a test of the failure path)."""
         check(_lib().sc_lbm_set_wait(self._h, int(limit_ns), int(withhold_cta)))
 
 

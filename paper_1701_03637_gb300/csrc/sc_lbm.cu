@@ -2218,10 +2218,15 @@ const char* sc_lbm_kernel_name(sc_lbm* h) {
 int sc_lbm_set_wait(sc_lbm* h, int64_t limit_ns, int32_t withhold_cta) {
   if (!h) return fail(SC_EINVAL, "NULL handle");
   if (limit_ns <= 0) return fail(SC_EINVAL, "limit_ns must be > 0");
-  if (withhold_cta < -1 || (h->persist && withhold_cta >= h->pcx * h->pcy))
+  // on a step without progress waits the hook has no effect
+  if (withhold_cta < -1 || ((h->persist || h->lay.shift) && withhold_cta >= h->grid))
     return fail(SC_EINVAL, "withhold_cta out of range");
   h->wait_limit_ns = limit_ns;
   h->withhold = withhold_cta;
+  if (h->lay.shift && h->graph) {  // the captured launches hold the old limit
+    cudaGraphExecDestroy(h->graph);
+    h->graph = nullptr;
+  }
   return SC_OK;
 }
 

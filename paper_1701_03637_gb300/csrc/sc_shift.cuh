@@ -63,6 +63,7 @@ struct ShiftArgs {
   unsigned* done;       // chunks finished, per tile column
   int* err;             // set to 3 when a wait gave up
   long long limit_ns;   // of a wait
+  int withhold;         // CTA that reports no finished chunk (-1: none)
 };
 
 // Copies `n16` 16-byte pieces (two planes) of each of the Q arrays and clears the column counters.
@@ -118,7 +119,7 @@ __global__ void __launch_bounds__(TX * TY, 512 / (TX * TY))
       t.evap = 0.0;
     }
     __syncthreads();  // the item's last reads and stores, and the next item's number
-    if (ok && threadIdx.x == 0) st_release_u32(a.done + col, (unsigned)k + 1u);
+    if (ok && threadIdx.x == 0 && (int)blockIdx.x != a.withhold) st_release_u32(a.done + col, (unsigned)k + 1u);
   }
 }
 
@@ -189,7 +190,7 @@ cudaError_t launch_shift(sc_lbm* h, cudaStream_t st) {
   const int n16 = (int)(kGhosts * plane / E);
   unsigned* done = (unsigned*)h->flags();
   k_shift_begin<<<grid_for((long long)Q * n16, 1024), 256, 0, st>>>((const int4*)from, (int4*)to, h->L.np / E, n16, done, l.cols);
-  const ShiftArgs a{l.cols_x, l.cols / l.cols_x, h->nitems, (int)l.nslots, down, h->next(), done, h->h_err, h->wait_limit_ns};
+  const ShiftArgs a{l.cols_x, l.cols / l.cols_x, h->nitems, (int)l.nslots, down, h->next(), done, h->h_err, h->wait_limit_ns, h->withhold};
   k_shift<64, 4, S><<<h->grid, 256, shift_smem<S>(h->L), st>>>(h->L, src, (T*)h->pop(1 - h->cur), h->evap(), a,
                                                                h->maps[h->cur]);
   return cudaGetLastError();

@@ -157,7 +157,7 @@ typedef struct sc_diag {
   double radius;                  /* (3 V / 4 pi)^(1/3), V = number of sites with rho^r > rho^b */
   int64_t droplet_sites;          /* V */
   int32_t status;                 /* SC_OK, SC_ENONFINITE, SC_ESINKNEG, or SC_ETIMEOUT after a
-                                     persistent in-place launch gave up a wait */
+                                     step gave up a wait (see sc_lbm_set_wait) */
   int32_t reserved;
 } sc_diag;
 
@@ -269,7 +269,8 @@ const char* sc_lbm_kernel_name(sc_lbm* h);
    the shifted one (default 2 s; SC_LAYOUT_AA), from the next step on, and a test hook: CTA
    withhold_cta (-1: none; below the CTA count of sc_lbm_launch_info) never reports its
    progress, so that its neighbours' waits run out after limit_ns. A wait that runs out ends
-   the step early; the state is then undefined, sc_lbm_sync returns SC_ETIMEOUT and
+   the step early; the state is then undefined, sc_lbm_sync, _read_fields, _read_populations,
+   _profile and _flux_profile return SC_ETIMEOUT (their output is that undefined state) and
    diagnostics report status SC_ETIMEOUT until a state is loaded (sc_lbm_init, _init_fields,
    _write_populations). Nothing waits without a limit, so the device stays usable. Steps
    without progress waits ignore both. No counterpart in the paper. */

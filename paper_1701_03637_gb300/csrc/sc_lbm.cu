@@ -732,7 +732,8 @@ __device__ __forceinline__ unsigned long long splitmix64_at(unsigned long long s
 template <class S>
 __global__ void k_load(const LatDev L, typename S::T* __restrict__ dst, long long s0, long long s1, int mode,
                        const float* __restrict__ f_in, long long f_stride, const float* __restrict__ rho_in,
-                       long long rho_stride, const ShapeDev sh, long long nsites) {
+                       long long rho_stride, const ShapeDev sh, long long nsites, int* __restrict__ err) {
+  if (blockIdx.x == 0 && threadIdx.x == 0) *err = 0;  // in the stream's order: steps before this load may still set it
   for (long long s = s0 + blockIdx.x * (long long)blockDim.x + threadIdx.x; s < s1;
        s += (long long)gridDim.x * blockDim.x) {
     int x, y, z;
@@ -1042,7 +1043,7 @@ struct sc_lbm {
   double evap_offset;  // evaporated mass restored by sc_lbm_set_counters
   double* h_diag;      // pinned
   double* h_evap;      // pinned
-  int* h_err;          // pinned, written by a step whose copies did not land in time
+  int* h_err;          // pinned, set by a step whose copies (3) or whose neighbours (4) did not come in time
   CUtensorMap maps[2]; // of the two population buffers, with the tile's box (staged rows)
   int grid;  // CTAs of the persistent step (in place: of k_aa_collide)
   int grid_psi;  // CTAs of k_aa_psi
@@ -1408,11 +1409,15 @@ int launch_persist(sc_lbm* h, int K, cudaStream_t st) {
   return SC_OK;
 }
 
-// After the stream is synchronised: SC_ETIMEOUT when a wait of the persistent step or of a
-// step's plane copies gave up (the lattice's state is then undefined until it is loaded again).
-int persist_status(sc_lbm* h) {
-  if (*(volatile int*)h->h_err != 0)
-    return fail(SC_ETIMEOUT, "a step's copies of a plane did not land in time; load a state to continue");
+// After the stream is synchronised: SC_ETIMEOUT when a wait of the persistent or the shifted step
+// or of a step's plane copies gave up (the lattice's state is then undefined until it is loaded
+// again). Every call that hands the state to the host ends with it.
+int wait_status(sc_lbm* h) {
+  const int e = *(volatile int*)h->h_err;
+  if (e != 0)
+    return fail(SC_ETIMEOUT, "%s; load a state to continue",
+                e == 4 ? "a wait of the shifted in-place step for its neighbours gave up"
+                       : "a step's copies of a plane did not land in time");
   if (!h->persist) return SC_OK;
   int v = 0;
   CK(cudaMemcpyAsync(&v, h->err(), sizeof(int), cudaMemcpyDeviceToHost, h->stream));
@@ -1474,7 +1479,7 @@ int launch_load(sc_lbm* h, long long s0, long long s1, int mode, const float* f,
                 long long rs, const ShapeDev& sh) {
   // the pull reads the current buffer, so the load writes it
   k_load<S><<<grid_for(s1 - s0, 256), 256, 0, h->stream>>>(h->L, (typename S::T*)h->pop(h->cur), s0, s1, mode, f, fs,
-                                                            rho, rs, sh, (long long)h->p.nx * h->p.ny * h->L.nzg);
+                                                            rho, rs, sh, (long long)h->p.nx * h->p.ny * h->L.nzg, h->h_err);
   CK(cudaGetLastError());
   return SC_OK;
 }
@@ -1482,12 +1487,8 @@ int launch_load(sc_lbm* h, long long s0, long long s1, int mode, const float* f,
 int load(sc_lbm* h, long long s0, long long s1, int mode, const float* f, long long fs, const float* rho,
          long long rs, const ShapeDev& sh) {
   // every caller loads the whole lattice; in place it is written in the even form
-  // (the two-lattice pull's slots); a new state clears the persistent step's error
+  // (the two-lattice pull's slots); a new state clears the error words
   if (h->lay.aa) h->cur = 0;
-  if (*(volatile int*)h->h_err != 0) {
-    CK(cudaStreamSynchronize(h->stream));
-    *h->h_err = 0;
-  }
   if (h->persist) CK(cudaMemsetAsync(h->err(), 0, sizeof(int), h->stream));
   switch (h->p.storage) {
     case SC_STORAGE_F16: return launch_load<StF16>(h, s0, s1, mode, f, fs, rho, rs, sh);
@@ -1732,7 +1733,7 @@ int sc_lbm_set_stream(sc_lbm* h, void* stream) {
 int sc_lbm_sync(sc_lbm* h) {
   if (!h) return fail(SC_EINVAL, "NULL handle");
   CK(cudaStreamSynchronize(h->stream));
-  return persist_status(h);
+  return wait_status(h);
 }
 
 int sc_lbm_init(sc_lbm* h, const sc_init* in) {
@@ -1867,7 +1868,7 @@ int sc_lbm_read_fields(sc_lbm* h, float* rr, float* rb) {
   CK(cudaMemcpyAsync(rb, h->stage() + h->lay.stage_n, sizeof(float) * h->lay.nsites, cudaMemcpyDeviceToHost,
                      h->stream));
   CK(cudaStreamSynchronize(h->stream));
-  return SC_OK;
+  return wait_status(h);
 }
 
 int sc_lbm_read_populations(sc_lbm* h, double* f) {
@@ -1885,7 +1886,7 @@ int sc_lbm_read_populations(sc_lbm* h, double* f) {
     for (int k = 0; k < 2 * Q; ++k)
       for (long long o = 0; o < m; ++o) f[(long long)k * n + s0 + o] = (double)tmp[(size_t)k * m + o];
   }
-  return SC_OK;
+  return wait_status(h);
 }
 
 int sc_lbm_write_populations(sc_lbm* h, const double* f) {
@@ -1955,7 +1956,7 @@ int sc_lbm_flux_profile(sc_lbm* h, double* j) {
       for (int k = 0; k < ns; ++k) acc += h->h_diag[((size_t)z * ns + k) * kDiagFields + d];
       j[(size_t)d * nz + z] = acc / nxy;
     }
-  return SC_OK;
+  return wait_status(h);
 }
 
 int sc_lbm_profile(sc_lbm* h, double* phi) {
@@ -1970,7 +1971,7 @@ int sc_lbm_profile(sc_lbm* h, double* phi) {
     for (int k = 0; k < ns; ++k) acc += h->h_diag[((size_t)z * ns + k) * kDiagFields + 2];
     phi[z] = acc / nxy;
   }
-  return SC_OK;
+  return wait_status(h);
 }
 
 int sc_lbm_diagnostics(sc_lbm* h, sc_diag* d) {
@@ -2015,7 +2016,7 @@ int sc_lbm_diagnostics(sc_lbm* h, sc_diag* d) {
   }
   d->status = nonfinite > 0.0 ? SC_ENONFINITE : (sinkneg > 0.0 ? SC_ESINKNEG : SC_OK);
   if (!std::isfinite(d->mass_r) || !std::isfinite(d->mass_b)) d->status = SC_ENONFINITE;
-  if (persist_status(h) == SC_ETIMEOUT) d->status = SC_ETIMEOUT;
+  if (wait_status(h) == SC_ETIMEOUT) d->status = SC_ETIMEOUT;
   return SC_OK;
 }
 
@@ -2070,6 +2071,8 @@ int sc_lbm_tune(sc_lbm* h, int32_t trials, int32_t* tile, int32_t* zchunk) {
   LaunchCfg best;
   int rc = plan_launch(&h->p, h->lay, h->lay.tile, h->p.zchunk, &best);  // the current choice
   if (rc) return rc;
+  CK(cudaStreamSynchronize(h->stream));
+  const int before = *(volatile int*)h->h_err;  // of the state, which the trials leave as it is
   float best_ms = 1e30f;
   cudaEvent_t e0, e1;
   CK(cudaEventCreate(&e0));
@@ -2100,6 +2103,11 @@ int sc_lbm_tune(sc_lbm* h, int32_t trials, int32_t* tile, int32_t* zchunk) {
       if (e == cudaSuccess) e = cudaEventRecord(e1, h->stream);
       if (e == cudaSuccess) e = cudaEventSynchronize(e1);
       if (e != cudaSuccess) { rc = fail(SC_ECUDA, "tuning trial failed: %s", cudaGetErrorString(e)); break; }
+      if (*(volatile int*)h->h_err != before) {
+        *h->h_err = before;
+        rc = fail(SC_ETIMEOUT, "a tuning trial's copies of a plane did not land in time");
+        break;
+      }
       float ms = 0.f;
       cudaEventElapsedTime(&ms, e0, e1);
       if (ms < best_ms) { best_ms = ms; best = c; }

@@ -61,7 +61,7 @@ struct ShiftArgs {
   bool down;
   unsigned* next;       // claim counter, 0 between launches
   unsigned* done;       // chunks finished, per tile column
-  int* err;             // set to 3 when a wait gave up
+  int* err;             // set to 3 when a plane's copies, to 4 when a neighbour's chunk did not come in time
   long long limit_ns;   // of a wait
   int withhold;         // CTA that reports no finished chunk (-1: none)
 };
@@ -106,13 +106,16 @@ __global__ void __launch_bounds__(TX * TY, 512 / (TX * TY))
         while (got && ld_acquire_u32(d) < (unsigned)k) got = (long long)(global_ns() - t0) <= a.limit_ns;
       }
     }
-    if (__syncthreads_or(!got)) ok = false;
+    if (__syncthreads_or(!got)) {
+      ok = false;
+      if (threadIdx.x == 0) *a.err = 4;
+    }
     if (ok) {
       t.setup(bx, by);
       const int c = a.down ? a.nch - 1 - k : k;
       ok = t.run((int)((long long)c * L.nz / a.nch), (int)((long long)(c + 1) * L.nz / a.nch), a.down);
+      if (!ok && threadIdx.x == 0) *a.err = 3;
     }
-    if (!ok && threadIdx.x == 0) *a.err = 3;
     if (L.geometry != 0 && __syncthreads_or(t.evap != 0.0)) {
       const double e = t.block_evap();
       if (threadIdx.x == 0) atomicAdd(evap_cum + it % a.nslots, e);

@@ -286,8 +286,10 @@ int sc_lbm_set_wait(sc_lbm* h, int64_t limit_ns, int32_t withhold_cta);
    of two, dividing nx, for which a tile grid fits); k >= 1 uses k bands (k must
    divide nx into bands of at least 2 sites) and re-plans the tile grid for the
    following steps. *bands (may be NULL) receives the count in use, 0 for a lattice
-   without the persistent step. SC_EINVAL for a request on such a lattice, for a k that
-   does not divide nx, or when no tile grid fits k bands (the previous plan is kept).
+   without the persistent step. An automatic lattice of the shifted step whose planes have
+   2^17 sites or more takes the persistent step with the first accepted request. SC_EINVAL
+   for a request on any other lattice without that step, for a k that does not divide nx,
+   or when no tile grid fits k bands (nothing has changed then).
    Tuning and test hook; no counterpart in the paper. */
 int sc_lbm_persist_bands(sc_lbm* h, int32_t request, int32_t* bands);
 /* Bytes one sc_lbm_diagnostics / sc_lbm_profile call copies device-to-host. */

@@ -670,7 +670,8 @@ __device__ __align__(256) double g_noalloc_scratch[kNoAllocScratch];
 
 __global__ void k_diag_finish(const double* __restrict__ part, int nz, int nsplit, double nxy, int wall_z0,
                               int wall_z1, const double* __restrict__ evap_slots, long long nslots,
-                              double evap_offset, const int* __restrict__ persist_err, double* __restrict__ out) {
+                              double evap_offset, const int* __restrict__ persist_err, const int* __restrict__ err,
+                              double* __restrict__ out) {
   if (blockIdx.x != 0 || threadIdx.x != 0) return;
   double mass_r = 0.0, mass_b = 0.0, pending = 0.0, count = 0.0, nonfinite = 0.0, sinkneg = 0.0;
   const int z0 = wall_z1 > wall_z0 ? wall_z1 : 0;
@@ -707,7 +708,7 @@ __global__ void k_diag_finish(const double* __restrict__ part, int nz, int nspli
   out[6] = count;
   const bool bad = nonfinite > 0.0 || !isfinite(mass_r) || !isfinite(mass_b);
   out[7] = bad ? (double)SC_ENONFINITE : (sinkneg > 0.0 ? (double)SC_ESINKNEG : (double)SC_OK);
-  if (persist_err && *persist_err != 0) out[7] = (double)SC_ETIMEOUT;
+  if ((persist_err && *persist_err != 0) || *err != 0) out[7] = (double)SC_ETIMEOUT;
 }
 
 // Initial / restored state: canonical populations of sites [s0, s1) from
@@ -2040,7 +2041,7 @@ int sc_lbm_diagnostics_noalloc(sc_lbm* h, double* out_dev) {
   if (rc) return rc;
   k_diag_finish<<<1, 1, 0, h->stream>>>(part, h->p.nz, h->lay.diag_nsplit, (double)h->p.nx * h->p.ny, h->L.wall_z0,
                                         h->L.wall_z1, h->evap(), h->lay.nslots, h->evap_offset,
-                                        h->persist ? h->err() : h->h_err, out_dev);
+                                        h->persist ? h->err() : nullptr, h->h_err, out_dev);
   CK(cudaGetLastError());
   return SC_OK;
 }
@@ -2242,21 +2243,9 @@ int sc_lbm_persist_bands(sc_lbm* h, int32_t request, int32_t* bands) {
   if (!h) return fail(SC_EINVAL, "NULL handle");
   if (request < -1) return fail(SC_EINVAL, "request must be -1, 0 or a band count");
   if (request >= 0) {
-    if (h->lay.shift && large_planes(&h->p)) {  // its persistent plan, where one exists
-      const Layout lay = h->lay;
-      const int cur = h->cur;
-      int rc = shift_to_persist(h);
-      if (rc) return rc;
-      rc = plan_aa(h);
-      if (rc || !h->persist) {
-        h->lay = lay;
-        h->cur = cur;
-        h->persist = false;
-        const int back = plan_shift(h);
-        if (rc || back) return rc ? rc : back;
-      }
-    }
-    if (!h->persist) return fail(SC_EINVAL, "the lattice does not use the persistent in-place step");
+    // a shifted lattice of large planes changes over, once nothing can refuse the request any more
+    const bool shifted = h->lay.shift && large_planes(&h->p);
+    if (!h->persist && !shifted) return fail(SC_EINVAL, "the lattice does not use the persistent in-place step");
     if (request > 1 && (h->p.nx % request != 0 || h->p.nx / request < 2))
       return fail(SC_EINVAL, "%d bands must divide nx = %d into bands of at least 2 sites", request, h->p.nx);
     const int old = h->pband_req;
@@ -2264,9 +2253,16 @@ int sc_lbm_persist_bands(sc_lbm* h, int32_t request, int32_t* bands) {
     if (!plan_persist(h)) {
       const char* why = h->persist_why;
       h->pband_req = old;
-      plan_persist(h);  // the previous plan, which fitted
-      apply_persist(h);
+      if (h->persist) plan_persist(h);  // the previous plan, which fitted
       return fail(SC_EINVAL, "no persistent plan with %d bands: %s", request, why);
+    }
+    if (shifted) {
+      const int rc = shift_to_persist(h);
+      if (rc) {
+        h->pband_req = old;
+        return rc;
+      }
+      h->persist = true;
     }
     apply_persist(h);
   }

@@ -1813,7 +1813,7 @@ int sc_lbm_step(sc_lbm* h, int64_t nsteps) {
     h->step += nsteps;
     return SC_OK;
   }
-  if (h->rcta > 0 && nsteps > 1) {  // a single step is not worth the way into shared memory and back
+  if (resident_takes(h, nsteps)) {
     int rc = launch_resident(h, nsteps);
     if (rc) return rc;
     h->step += nsteps;
@@ -2210,7 +2210,7 @@ int sc_lbm_launch_count(sc_lbm* h, int64_t nsteps, int64_t* launches) {
   if (!h || !launches) return fail(SC_EINVAL, "NULL argument");
   if (nsteps < 0) return fail(SC_EINVAL, "nsteps must be >= 0");
   if (h->persist) *launches = (nsteps + persist_max_steps(h) - 1) / persist_max_steps(h);
-  else if (h->rcta > 0 && nsteps > 1) *launches = (nsteps + kResidentMaxSteps - 1) / kResidentMaxSteps;
+  else if (resident_takes(h, nsteps)) *launches = (nsteps + kResidentMaxSteps - 1) / kResidentMaxSteps;
   else *launches = h->lay.aa || h->lay.shift ? 2 * nsteps : nsteps;
   return SC_OK;
 }

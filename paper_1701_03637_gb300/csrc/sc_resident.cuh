@@ -13,9 +13,6 @@
 // these form that plane's Psi from its populations (the owner's arithmetic, so its bits): Psi
 // is then shared within the CTA and the first cluster barrier is a CTA barrier: 100 film steps
 // with diagnostics and read-out 168 -> 155 us.
-// A call of one step takes the two-lattice kernel instead: getting into shared memory and back
-// costs more than the step (one step of 20^3 FP32 16.7 against 8.5 us, of 4x4x128 10.5 against 8.5;
-// two steps 20.8 against 16.8 and 12.1 against 16.7).
 // The addresses of the 19 sources are the same in every step and stay in registers (a
 // population next to a wall is the site's own opposite one, and a solid neighbour's Psi a
 // cell that holds 0), so a step has no index arithmetic. Values are rounded to the
@@ -234,6 +231,18 @@ void plan_resident(sc_lbm* h) {
     cudaGetLastError();
     h->rcta = 0;
   }
+}
+
+// Whether a call of nsteps steps takes the resident launch. A single step is not worth the way into
+// shared memory and back (us for one step, resident / two-lattice: 20^3 FP32 16.7 / 8.5, 4x4x128 10.5 /
+// 8.5; for two steps 20.8 / 16.8 and 12.1 / 16.7), unless the two-lattice tiles of 8 x 4 sites are
+// nearly empty and many (1x1x100 16.6 / 15.9, 1x1x1000 18.3 / 26.5, 1x1x8000 19.9 / 67.7, 1x8x1000
+// 19.7 / 25.7, 1x64x100 18.8 / 22.6, 2x2x2000 20.0 / 21.2; against 8x1x1000 19.8 / 17.0, 2x3x1300
+// 19.9 / 18.1; with the host's wait, 6 us).
+bool resident_takes(const sc_lbm* h, int64_t nsteps) {
+  if (h->rcta == 0 || nsteps != 1) return h->rcta > 0;
+  const long long lanes = 32LL * ((h->p.nx + 7) / 8) * ((h->p.ny + 3) / 4) * h->p.nz;
+  return lanes >= 16000 && lanes >= 8 * h->lay.nsites;
 }
 
 // nsteps steps in place on the current buffer.

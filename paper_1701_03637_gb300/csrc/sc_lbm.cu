@@ -67,7 +67,9 @@ int wrap_host(int v, int n) { return ((v % n) + n) % n; }
 // and then from L2 by its neighbours, whatever each CTA's speed. (Dealt out round-robin,
 // slower CTAs fell further behind with every item.) CTA b's first
 // item is item b. The counter wraps to 0 with the last claim of the launch (items past the
-// first per CTA, and one failing claim per CTA).
+// first per CTA, and one failing claim per CTA). Launches with a sink and more items than
+// evaporated-mass slots (chosen chunk lengths) deal them out all the same: next is null and
+// nslots the grid.
 template <int TX, int TY, class S, bool Rows>
 __global__ void __launch_bounds__(TX * TY, (512 / (TX * TY)) > 1 ? 512 / (TX * TY) : 1)
     k_step(const LatDev L, const typename S::T* __restrict__ src, typename S::T* __restrict__ dst,
@@ -82,7 +84,8 @@ __global__ void __launch_bounds__(TX * TY, (512 / (TX * TY)) > 1 ? 512 / (TX * T
   int turn = 0;
   bool ok = true;
   for (int it = (int)blockIdx.x; it < nitems; it = s_it[turn ^= 1]) {
-    if (threadIdx.x == 0) s_it[turn ^ 1] = G + (int)atomicInc(next, (unsigned)nitems - 1u);  // one item ahead
+    if (threadIdx.x == 0)  // one item ahead
+      s_it[turn ^ 1] = G + (next ? (int)atomicInc(next, (unsigned)nitems - 1u) : it);
     if (ok) {
       const int4 w = items[it];  // tile column, first plane, end plane, downward
       t.setup(w.x % cols_x, w.x / cols_x);
@@ -91,7 +94,8 @@ __global__ void __launch_bounds__(TX * TY, (512 / (TX * TY)) > 1 ? 512 / (TX * T
     }
     if (L.geometry != 0 && __syncthreads_or(t.evap != 0.0)) {
       const double e = t.block_evap();
-      // a slot per item; launches with more items than slots share them
+      // a slot per item, or per CTA of dealt items, so that the order of the sums does not depend on
+      // which CTA claims what
       if (threadIdx.x == 0) atomicAdd(evap_cum + it % nslots, e);
       t.evap = 0.0;
     }
@@ -817,9 +821,10 @@ constexpr size_t step_smem(const LatDev& L) {
 
 template <int TX, int TY, class S, bool Rows>
 cudaError_t launch_step(const StepArgs& a) {
+  const bool dealt = a.L.geometry != 0 && a.nitems > a.nslots;
   k_step<TX, TY, S, Rows><<<a.G, TX * TY, step_smem<TX, TY, S, Rows>(a.L), a.st>>>(
-      a.L, (const typename S::T*)a.src, (typename S::T*)a.dst, a.evap, a.nslots, a.cols_x, a.items, a.nitems, a.next, a.map,
-      a.err);
+      a.L, (const typename S::T*)a.src, (typename S::T*)a.dst, a.evap, dealt ? a.G : a.nslots, a.cols_x, a.items, a.nitems,
+      dealt ? nullptr : a.next, a.map, a.err);
   return cudaGetLastError();
 }
 
@@ -1143,7 +1148,9 @@ int plan_launch(const sc_params* p, const Layout& l, int tile, int zchunk, Launc
     best_nch = (nz + zchunk - 1) / zchunk;
   } else {
     double best = 1e300;
-    for (long long nch = 1; nch <= nz && cols * nch <= l.cap_items; ++nch) {
+    // with a sink, no more items than evaporated-mass slots (k_step; costs under 5% of this estimate)
+    const long long most = p->geometry != 0 ? std::max(l.nslots, cols) : l.cap_items;
+    for (long long nch = 1; nch <= nz && cols * nch <= most; ++nch) {
       const long long rounds = (cols * nch + slots - 1) / slots;
       const double cost = (double)rounds * ((double)((nz + nch - 1) / nch) + 2.0);
       if (cost < best * (1.0 - 1e-9)) { best = cost; best_nch = nch; }

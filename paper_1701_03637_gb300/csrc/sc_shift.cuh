@@ -57,7 +57,7 @@ __device__ __forceinline__ void st_release_u32(unsigned* p, unsigned v) {
 }
 
 struct ShiftArgs {
-  int cols_x, cols_y, nch, nslots;
+  int cols_x, cols_y, nch;
   bool down;
   unsigned* next;       // claim counter, 0 between launches
   unsigned* done;       // chunks finished, per tile column
@@ -118,7 +118,7 @@ __global__ void __launch_bounds__(TX * TY, 512 / (TX * TY))
     }
     if (L.geometry != 0 && __syncthreads_or(t.evap != 0.0)) {
       const double e = t.block_evap();
-      if (threadIdx.x == 0) atomicAdd(evap_cum + it % a.nslots, e);
+      if (threadIdx.x == 0) atomicAdd(evap_cum + col, e);  // the column's chunks follow one another
       t.evap = 0.0;
     }
     __syncthreads();  // the item's last reads and stores, and the next item's number
@@ -193,7 +193,7 @@ cudaError_t launch_shift(sc_lbm* h, cudaStream_t st) {
   const int n16 = (int)(kGhosts * plane / E);
   unsigned* done = (unsigned*)h->flags();
   k_shift_begin<<<grid_for((long long)Q * n16, 1024), 256, 0, st>>>((const int4*)from, (int4*)to, h->L.np / E, n16, done, l.cols);
-  const ShiftArgs a{l.cols_x, l.cols / l.cols_x, h->nitems, (int)l.nslots, down, h->next(), done, h->h_err, h->wait_limit_ns, h->withhold};
+  const ShiftArgs a{l.cols_x, l.cols / l.cols_x, h->nitems, down, h->next(), done, h->h_err, h->wait_limit_ns, h->withhold};
   k_shift<64, 4, S><<<h->grid, 256, shift_smem<S>(h->L), st>>>(h->L, src, (T*)h->pop(1 - h->cur), h->evap(), a,
                                                                h->maps[h->cur]);
   return cudaGetLastError();

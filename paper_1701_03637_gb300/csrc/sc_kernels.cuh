@@ -773,8 +773,8 @@ struct TileRows {
 
   const LatDev& L;
   Smem& sm;
-  const T* __restrict__ src;
-  T* __restrict__ dst;
+  const T* src;  // Shift: src and dst overlap
+  T* dst;
   const CUtensorMap* map;
   int tx, ty, x, y, hx, hy, hlx, hly, x0, y0;
   int tw, th;                  // the tile's sites in x and y
@@ -915,7 +915,9 @@ struct TileRows {
   __device__ __forceinline__ float2 pulled(int ly, int lx, bool sol_m, bool sol_p, Index s) const {
     constexpr int ez = dir_z(I);
     if (ez != 0 && (ez > 0 ? sol_m : sol_p)) {
-      return ld<S>(src + (long long)opp(I) * L.np + s, wgt(I));
+      const T* p = src + (long long)opp(I) * L.np + s;
+      if constexpr (Shift) return ldcg<S>(p, wgt(I));  // other CTAs of the launch write this memory later on
+      else return ld<S>(p, wgt(I));
     }
     return staged<I>(ly, lx);
   }

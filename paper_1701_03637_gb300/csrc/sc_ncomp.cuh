@@ -159,10 +159,13 @@ __global__ void __launch_bounds__(kNT) k_n_step(const NDev D, const float* __res
 // The same step in two launches, a site per thread: Psi of every component into an array, then
 // the rest with Psi from there. No halo is formed twice and no CTA waits for another's plane,
 // but every population is read twice: for lattices whose two buffers stay in the L2. Bound by
-// the latency and the issue of its loads. Per step, marched against in two launches: 64^3 of 2
-// components 30.8 / 22.6 us, of 3 39.0 / 34.8; 48^3 of 3 22.6 / 20.5; beyond the L2 80^3 of 3
-// 75.8 / 81.9. With 4 components the marched step, which shares its index arithmetic among
-// them, stays ahead (32^3 12.3 / 14.2, 64^3 53.3 / 55.3).
+// the latency and the issue of its loads. us per step, marched / in two launches: 2 components 8^3
+// 10.5 / 8.5, 16^3 10.6 / 8.5, 24^3 11.5 / 10.5, 32^3 10.6 / 10.5, 40^3 16.8 / 14.6, 64^3 31.1 / 22.8,
+// 72^3 47.5 / 39.5; 3 components 16^3 12.5 / 9.5, 24^3 12.6 / 10.5, 32^3 12.5 / 11.5, 40^3 22.8 / 16.7,
+// 48^3 22.8 / 20.2, 64^3 39.6 / 35.0, 24x24x80 14.7 / 14.6, 80x24x24 16.7 / 12.6, 33x50x70 37.1 / 26.0;
+// a call of one step is 1 to 17 us shorter too. Beyond the L2 80^3 of 3 75.8 / 81.9. With 4
+// components the marched step, which shares its index arithmetic among them, stays ahead
+// (32^3 12.3 / 14.2, 64^3 53.3 / 55.3).
 constexpr int kNSiteY = 4;  // rows of 32 sites per CTA
 constexpr size_t kNSitesBytes = kL2Bytes;
 template <int NC>
@@ -294,11 +297,7 @@ cudaError_t n_sites_launch(const NDev& D, const float* src, float* dst, float* p
   return cudaGetLastError();
 }
 cudaError_t n_sites_dispatch(int nc, const NDev& D, const float* src, float* dst, float* psi, cudaStream_t st) {
-  switch (nc) {
-    case 2: return n_sites_launch<2>(D, src, dst, psi, st);
-    case 3: return n_sites_launch<3>(D, src, dst, psi, st);
-    default: return n_sites_launch<4>(D, src, dst, psi, st);
-  }
+  return nc == 2 ? n_sites_launch<2>(D, src, dst, psi, st) : n_sites_launch<3>(D, src, dst, psi, st);
 }
 
 cudaError_t n_step_dispatch(int nc, const NDev& D, const float* src, float* dst, int cols_x, int cols, int nch,

@@ -50,7 +50,8 @@ extern "C" {
 #define SC_ENOMEM (-2)      /* device or host allocation failed, or caller buffer too small */
 #define SC_ECUDA (-3)       /* a CUDA runtime call failed (message has the CUDA error string) */
 #define SC_ENONFINITE (-4)  /* diagnostics found a NaN/Inf density */
-#define SC_ETIMEOUT (-5)    /* a bounded device-side wait gave up */
+#define SC_ETIMEOUT (-5)    /* a bounded device-side wait gave up: for neighbours (in place) or for a
+                               plane's copies (staged rows) */
 #define SC_ESINKNEG (-6)    /* a sink site had rho^r + rho^b < rho_H (negative complement) */
 
 #define SC_GEOM_PERIODIC 0      /* no sink */
@@ -63,15 +64,21 @@ extern "C" {
 #define SC_STORAGE_F16_SCALED 3 /* FP16 of f_i / w_i (about rho: the same relative spacing in liquid
                                    and vapour; not in the paper), FP32 arithmetic */
 
-#define SC_STAGING_AUTO 0       /* staged rows where nx allows, else per-thread pulls */
-#define SC_STAGING_THREAD 1     /* each thread copies its site's 38 pulls (any nx) */
-#define SC_STAGING_ROWS 2       /* the CTA copies the tile's source rows as 16-byte chunks
+#define SC_STAGING_AUTO 0       /* the form measured fastest for the lattice: up to 8192 sites the
+                                   resident step (one cluster's shared memory holds the lattice
+                                   for all steps of a call, unless tile or zchunk is given), then
+                                   per-thread pulls, and staged rows on large lattices of wide
+                                   planes (nx a multiple of 2 for FP32, of 4 for 16-bit types);
+                                   in place see SC_LAYOUT_AA */
+#define SC_STAGING_THREAD 1     /* each thread copies its site's 19 pairs of populations (any nx) */
+#define SC_STAGING_ROWS 2       /* the CTA stages the tile's source rows, one TMA box per direction
                                    (nx a multiple of 4 for FP32, of 8 for FP16/BF16) */
 #define SC_STAGING_PERSISTENT 3 /* in place only (SC_LAYOUT_AA): one cooperative launch advances
                                    many steps, each CTA keeping one tile column and ordering its
                                    in-place writes against its neighbours' reads with bounded
-                                   progress waits (see SC_LAYOUT_AA). SC_STAGING_AUTO picks it
-                                   for in-place lattices when the device can keep one CTA per
+                                   progress waits (see SC_LAYOUT_AA). SC_STAGING_AUTO picks it for
+                                   in-place lattices of 2^17 sites per plane or more that do not
+                                   take the shifted step, when the device can keep one CTA per
                                    tile column resident; SC_STAGING_THREAD keeps the two-pass
                                    step. */
 
@@ -191,9 +198,11 @@ int sc_lbm_init(sc_lbm* h, const sc_init* in);
    then the sink reset. Synchronous. */
 int sc_lbm_init_fields(sc_lbm* h, const float* rho_r_host, const float* rho_b_host);
 
-/* Advance nsteps time steps (asynchronous). Each step is one fused launch
-   (stream + sink reset + densities + Psi + force + collision) with two lattices,
-   two launches in place (Psi, then the rest; SC_LAYOUT_AA). */
+/* Advance nsteps time steps (asynchronous). With two lattices each step is one fused launch
+   (stream + sink reset + densities + Psi + force + collision); lattices of the resident step
+   advance up to 4096 steps per launch in calls of two steps and more. In place
+   (SC_LAYOUT_AA) a step is two launches (Psi and the rest, or the shifted step and the copy
+   before it), or up to 1024 steps are one (the persistent step). */
 int sc_lbm_step(sc_lbm* h, int64_t nsteps);
 
 /* Canonical densities into caller buffers (nx*ny*nz floats each). */
@@ -244,10 +253,13 @@ int sc_lbm_flux_profile(sc_lbm* h, double* j_host);
    (sc_slab_create) are rejected with SC_EINVAL. */
 int sc_lbm_diagnostics_noalloc(sc_lbm* h, double* out_dev);
 
-/* Kernel configuration in use: tile extents, planes per CTA, grid size and the
-   staging (SC_STAGING_THREAD or SC_STAGING_ROWS). With SC_LAYOUT_AA: a row segment
-   of tile_x sites per CTA, tile_y = zchunk = 1, SC_STAGING_THREAD. Any output
-   pointer may be NULL. */
+/* Kernel configuration in use: tile extents, planes per work item, grid size and the
+   staging (SC_STAGING_THREAD or SC_STAGING_ROWS). With SC_LAYOUT_AA: the two-pass step
+   reports a row segment of tile_x sites per CTA, tile_y = zchunk = 1 and
+   SC_STAGING_THREAD, the shifted step its 64 x 4 tiles, planes per chunk and
+   SC_STAGING_ROWS, the persistent step its tiles and SC_STAGING_PERSISTENT. On a lattice
+   of the resident step the figures are those of the launch that single steps take. Any
+   output pointer may be NULL. */
 int sc_lbm_launch_info(sc_lbm* h, int32_t* tile_x, int32_t* tile_y, int32_t* zchunk, int64_t* ctas,
                        int32_t* staging);
 /* Autotuner of the step kernel: times `trials` launches of every tile shape x
@@ -255,7 +267,9 @@ int sc_lbm_launch_info(sc_lbm* h, int32_t* tile_x, int32_t* tile_y, int32_t* zch
    following steps; reports the tile (entry + 1 of sc_tile_list) and planes per
    CTA. Trial launches read the current state and write only the buffer the next
    step overwrites, booking their evaporated mass in scratch, so the state and
-   the bookkeeping are unchanged. Synchronous. No counterpart in the paper. With
+   the bookkeeping are unchanged. Synchronous. No counterpart in the paper. On a lattice
+   of the resident step it tunes the launch that single steps take; calls of two steps and
+   more stay with the resident launch, which is ahead of every tile there. With
    SC_LAYOUT_AA there is no spare buffer and one configuration: it times nothing
    and reports tile 0 and the current planes per CTA. */
 int sc_lbm_tune(sc_lbm* h, int32_t trials, int32_t* tile, int32_t* zchunk);
@@ -337,9 +351,10 @@ int sc_slab_unpack(sc_lbm* h, int32_t side, const void* in_dev);
    relaxation time tau[c]; g[c][cbar] is the coupling g^{c cbar} of Eq. (3) (the diagonal
    the self couplings). The common velocity is u' = sum_c (m^c / tau_c) /
    sum_c (rho^c / tau_c) and the shift tau_c F^c / rho^c, as for two components. FP32
-   populations, two lattices, one launch per step (tile columns of 32 x 8 sites marching
+   populations, two lattices; one launch per step (tile columns of 32 x 8 sites marching
    chunks of planes, Psi of every component in a shared ring, then pull + force +
-   collision). With two components and non-zero self couplings the populations are
+   collision), or, for two and three components whose two buffers fit the L2, two launches
+   with a thread per site (Psi of every component, then the rest; the same bits). With two components and non-zero self couplings the populations are
    bit-identical to sc_lbm_step's. */
 #define SC_MAX_COMP 4
 
@@ -365,7 +380,7 @@ int sc_ncomp_write_populations(sc_ncomp* h, const double* f_host);
 int sc_ncomp_init_fields(sc_ncomp* h, const float* rho_host);
 /* Canonical populations out (same layout; 0 at solid sites). Synchronous. */
 int sc_ncomp_read_populations(sc_ncomp* h, double* f_host);
-/* Advance nsteps steps (asynchronous, one launch per step). */
+/* Advance nsteps steps (asynchronous, one or two launches per step). */
 int sc_ncomp_step(sc_ncomp* h, int64_t nsteps);
 int sc_ncomp_sync(sc_ncomp* h);
 

@@ -94,7 +94,7 @@ __device__ __forceinline__ float2 vset<float2>(float a) { return make_float2(a, 
 // Everything a launch needs to know about one lattice.
 struct LatDev {
   int nx, ny, nz, nxny;
-  long long np;            // elements between consecutive (component, direction) arrays
+  long long np;            // pairs between consecutive direction arrays (N components: populations)
   float omega[2], tau[2];  // 1/tau and tau per component
   float G, rhoH;           // g of Eq. (3); imposed rho^r at sinks
   float Gs[2];             // self couplings g^{rr}, g^{bb} of Eq. (3) (0: the paper's two-component model)
@@ -457,7 +457,7 @@ __device__ __forceinline__ float2 shift_factor(float2 g, float2 tau, float2 rho,
 // Shifted-velocity BGK relaxation of a component (V = float) or of both (float2) at a
 // fluid site (Eqs. (1)-(3)): u_eq = u' + tau_c F^c / rho^c with F^c = -Psi^c(x) g A: g = G
 // and A = a^cbar = sum_i w_i Psi^cbar(x + e_i) e_i in the paper's two-component model,
-// g = 1 and A = sum_cbar g^{c cbar} a^cbar (coupled_sums) with self couplings.
+// g = 1 and A = sum_cbar g^{c cbar} a^cbar with self couplings.
 template <class V>
 __device__ __forceinline__ void relax_core(V om, V tau, V (&f)[Q], V rho, V ps, V g, const V (&A)[3],
                                            const float (&up)[3]) {
@@ -904,8 +904,8 @@ struct TileRows {
     return ok;
   }
 
-  // Population i of component c arriving at tile cell (lx, ly) (ly, lx in [-1, TY] x [-1, TX]):
-  // from the staged rows; next to a wall, a population whose source plane is solid
+  // Pair of direction I arriving at tile cell (lx, ly) (ly, lx in [-1, TY] x [-1, TX]):
+  // from the staged rows; next to a wall, a pair whose source plane is solid
   // is the site's (index s) own opposite one instead.
   template <int I>
   __device__ __forceinline__ float2 staged(int ly, int lx) const {

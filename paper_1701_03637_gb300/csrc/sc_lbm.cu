@@ -294,7 +294,7 @@ struct PersistTile {
   }
 
   // Psi of plane q (in [-1, nz]) over the tile and its halo ring into ring slot sa
-  // (and sb >= 0); the 38 loads of a cell are independent and in flight together.
+  // (and sb >= 0); the 19 loads of a cell are independent and in flight together.
   // Ring cell c is site (x0 + hx, y0 + hy), hx = c % RW - 1, hy = c / RW - 1
   // (periodic); cells past a ragged tile's halo are skipped.
   template <bool ODD>
@@ -552,6 +552,12 @@ __global__ void __launch_bounds__(kDiagThreads) k_diag(const LatDev L, const typ
 // Eq. (3) (periodic neighbours, Psi = 0 at solid sites, self couplings included),
 // evaluated in FP64 from the canonical populations; 0 at sink and solid sites.
 // Per (plane, split) partial sums of the three components go to `part`.
+//
+// FP64 at 1/64 of the FP32 rate and one chain of loads, sums and two exponentials per
+// neighbour bound it. Planes of up to kFluxPlane sites (one CTA per plane) form Psi of planes
+// z - 1, z, z + 1 once, a site per thread, in shared memory (SHARED) instead of at every one of
+// the 18 neighbours in turn: 10 steps of the 4x4x125 column with flux and read-out 146 -> 77 us.
+constexpr int kFluxPlane = 1000;  // under 48 KB of shared memory
 
 // FP64 densities of the canonical populations of site (x, y, z); returns its class.
 template <class S>
@@ -573,12 +579,6 @@ __device__ __forceinline__ int canonical_rho(const LatDev& L, const typename S::
   return cls;
 }
 
-//
-// FP64 at 1/64 of the FP32 rate and one chain of loads, sums and two exponentials per
-// neighbour bound it. Planes of up to kFluxPlane sites (one CTA per plane) form Psi of planes
-// z - 1, z, z + 1 once, a site per thread, in shared memory (SHARED) instead of at every one of
-// the 18 neighbours in turn: 10 steps of the 4x4x125 column with flux and read-out 146 -> 77 us.
-constexpr int kFluxPlane = 1000;  // under 48 KB of shared memory
 template <class S, bool SHARED>
 __global__ void __launch_bounds__(kDiagThreads) k_flux(const LatDev L, const typename S::T* __restrict__ src,
                                                        int nsplit, double* __restrict__ part, int odd, double G,
@@ -877,7 +877,7 @@ size_t elem_size(int storage) { return storage == SC_STORAGE_F32 ? 4 : 2; }
 
 struct Layout {
   int tile, tx, ty, cols_x, cols;
-  bool rows;                  // staged-rows step kernel (nx a multiple of a 16-byte chunk)
+  bool rows;                  // staged-rows step kernel (nx a multiple of 16 bytes of pairs)
   bool aa;                    // one population lattice in the AA forms (SC_LAYOUT_AA)
   bool shift;                 // one population lattice, shifted by `planes` planes each step (SC_LAYOUT_AA)
   int planes;
@@ -951,7 +951,7 @@ Layout make_layout(const sc_params* p) {
   l.off_psi = off;
   if (l.aa) off += align256((size_t)l.np * sizeof(float2));  // (Psi^r, Psi^b) per site
   else { l.off_pop[1] = off; off += pop; }
-  // the shifted step takes both regions as planes of the 38 arrays
+  // the shifted step takes both regions as planes of the 19 arrays
   l.planes = shift_planes(p, es, (long long)off, &l.np);
   if (l.planes > 0) {
     l.aa = false;
@@ -968,8 +968,8 @@ Layout make_layout(const sc_params* p) {
   // per site)
   l.cap_items = (long long)((p->nx + 7) / 8) * ((p->ny + 3) / 4) * p->nz;
   l.off_items = off; off += align256((size_t)l.cap_items * sizeof(int4));
-  // progress counters of the persistent in-place step (two per CTA), its error word, and
-  // the claim counter of the two-lattice step
+  // progress counters of the persistent in-place step (two per CTA) or of the shifted step (one per
+  // tile column), the persistent step's error word, and the claim counter of the other two
   l.off_flags = off; off += align256((size_t)2 * kMaxCtas * sizeof(unsigned long long) + 256);
   l.total = off;
   return l;
@@ -1066,7 +1066,7 @@ struct sc_lbm {
   const char* persist_why;   // why the persistent step was not planned
   bool slab;                 // z-slab of a larger lattice (sc_slab_create)
   int zmax;  // planes of the longest work item
-  int nitems;  // work items of a step (two lattices)
+  int nitems;  // work items of a step (two lattices), chunks of a step (shifted)
   int rcta, rsites;  // resident step: CTAs of its cluster (0: not used) and sites of each
   bool rplanes;      // whole planes per CTA, with threads for the plane on each side
   cudaGraphExec_t graph;

@@ -1598,6 +1598,45 @@ int noalloc_scratch(double** out) {
   return SC_OK;
 }
 
+// Whether a kernel on the current device can use the memory at p.
+bool on_device(const void* p, bool* yes) {
+  int dev = 0;
+  cudaPointerAttributes at{};
+  if (cudaGetDevice(&dev) != cudaSuccess) return false;
+  if (cudaPointerGetAttributes(&at, p) != cudaSuccess) cudaGetLastError();
+  *yes = at.type == cudaMemoryTypeDevice && at.device == dev;
+  return true;
+}
+
+// n sites of the Q arrays of pairs (r, b), np apart, to (or from) 2 * Q packed arrays of n
+// populations, component r's first. Bound by the memory; a face of 512^2 FP32 moves 2 * 160 MB.
+template <class E>
+struct alignas(2 * sizeof(E)) PopPair {
+  E r, b;
+};
+template <class E>
+__global__ void __launch_bounds__(256) k_faces(PopPair<E>* __restrict__ pairs, long long np, long long n,
+                                               E* __restrict__ packed, bool to_packed) {
+  for (long long t = blockIdx.x * 256LL + threadIdx.x; t < Q * n; t += gridDim.x * 256LL) {
+    const long long i = t / n, o = t - i * n;
+    PopPair<E>* p = pairs + i * np + o;
+    if (to_packed) {
+      const PopPair<E> v = *p;
+      packed[t] = v.r;
+      packed[Q * n + t] = v.b;
+    } else {
+      *p = PopPair<E>{packed[t], packed[Q * n + t]};
+    }
+  }
+}
+template <class E>
+int launch_faces(sc_lbm* h, int zl, long long n, void* packed, bool to_packed) {
+  PopPair<E>* pairs = (PopPair<E>*)h->pop(h->cur) + (long long)zl * h->L.nxny;
+  k_faces<E><<<grid_for(Q * n, 256), 256, 0, h->stream>>>(pairs, h->lay.np, n, (E*)packed, to_packed);
+  CK(cudaGetLastError());
+  return SC_OK;
+}
+
 template <class S>
 int launch_flux(sc_lbm* h) {
   dim3 grid(h->p.nz, h->lay.diag_nsplit);
@@ -1849,16 +1888,10 @@ int sc_lbm_read_fields_device(sc_lbm* h, float* rr, float* rb) {
   const long long n = h->lay.nsites;
   // the kernel writes the caller's arrays (rho^b at their distance from rho^r) where it can
   // reach them; overlapping, unaligned, host and other devices' memory takes a copy
-  int dev = 0;
-  CK(cudaGetDevice(&dev));
   const intptr_t apart = (intptr_t)rb - (intptr_t)rr, bytes = (intptr_t)(sizeof(float) * n);
   bool direct = (((uintptr_t)rr | (uintptr_t)rb) & 3) == 0 && (apart >= bytes || apart <= -bytes);
-  for (const float* p : {rr, rb}) {
-    cudaPointerAttributes at{};
-    if (!direct) break;
-    if (cudaPointerGetAttributes(&at, p) != cudaSuccess) cudaGetLastError();
-    direct = at.type == cudaMemoryTypeDevice && at.device == dev;
-  }
+  for (const float* p : {rr, rb})
+    if (direct && !on_device(p, &direct)) return fail(SC_ECUDA, "cudaGetDevice failed");
   if (direct) return canonical(h, 0, n, rr, apart / (intptr_t)sizeof(float), nullptr, 0);
   const int rc = canonical(h, 0, n, h->stage(), h->lay.stage_n, nullptr, 0);
   if (rc) return rc;
@@ -2185,17 +2218,22 @@ int sc_slab_info(sc_lbm* h, int32_t* z0, int32_t* z1, int32_t* ghosts, size_t* f
   return SC_OK;
 }
 
-// The kSlabGhosts planes starting at local plane zl of the current buffer, as 19
-// arrays of kSlabGhosts * nx * ny pairs each, to or from a packed device buffer.
+// The kSlabGhosts planes starting at local plane zl of the current buffer, as 2 * 19
+// arrays of kSlabGhosts * nx * ny populations each, to or from a packed device buffer.
+// Memory that the kernel cannot use (unaligned, not of this device) is reached by a copy
+// through the buffer that the next step overwrites.
 static int slab_copy(sc_lbm* h, int zl, void* packed, bool to_packed) {
-  const size_t ps = 2 * elem_size(h->p.storage);
-  const size_t run = (size_t)kSlabGhosts * h->p.nx * h->p.ny * ps;  // contiguous in each array
-  char* planes = (char*)h->pop(h->cur) + (size_t)zl * h->p.nx * h->p.ny * ps;
-  const size_t pitch = (size_t)h->lay.np * ps;
-  if (to_packed)
-    CK(cudaMemcpy2DAsync(packed, run, planes, pitch, run, Q, cudaMemcpyDeviceToDevice, h->stream));
-  else
-    CK(cudaMemcpy2DAsync(planes, pitch, packed, run, run, Q, cudaMemcpyDeviceToDevice, h->stream));
+  const size_t es = elem_size(h->p.storage);
+  const long long n = (long long)kSlabGhosts * h->L.nxny;
+  bool direct = false;
+  if (!on_device(packed, &direct)) return fail(SC_ECUDA, "cudaGetDevice failed");
+  direct = direct && (uintptr_t)packed % es == 0;
+  void* buf = direct ? packed : h->pop(1 - h->cur);
+  const size_t bytes = (size_t)2 * Q * n * es;
+  if (!direct && !to_packed) CK(cudaMemcpyAsync(buf, packed, bytes, cudaMemcpyDeviceToDevice, h->stream));
+  const int rc = es == 4 ? launch_faces<float>(h, zl, n, buf, to_packed) : launch_faces<uint16_t>(h, zl, n, buf, to_packed);
+  if (rc) return rc;
+  if (!direct && to_packed) CK(cudaMemcpyAsync(packed, buf, bytes, cudaMemcpyDeviceToDevice, h->stream));
   return SC_OK;
 }
 

@@ -75,8 +75,11 @@ __device__ __forceinline__ float vadd(float a, float b) { return __fadd_rn(a, b)
 __device__ __forceinline__ float vsub(float a, float b) { return __fsub_rn(a, b); }
 __device__ __forceinline__ float vmul(float a, float b) { return __fmul_rn(a, b); }
 __device__ __forceinline__ float vfma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
-// The builtins keep products and sums apart; add / mul.rn.f32x2 written as inline PTX are
-// contracted by the assembler (measured: 21% of random a b + c differed).
+// The compiler contracts a packed sum of a packed product that has no other use, written with
+// the builtins or in PTX, also as fma(c, 1, a b) (20.7% of 8.4M random a b + c differed from the
+// scalar operations); a sum or difference through fma by -1 is kept, and so is a product that a sum
+// and a difference share (none differed). So no product goes into vadd alone: vsub is the fma by
+// -1, relax_core's odd part is both added and subtracted, and StF16S decodes with scalar products.
 __device__ __forceinline__ float2 vadd(float2 a, float2 b) { return __fadd2_rn(a, b); }
 __device__ __forceinline__ float2 vmul(float2 a, float2 b) { return __fmul2_rn(a, b); }
 __device__ __forceinline__ float2 vfma(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
@@ -178,8 +181,9 @@ __device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
 // from global memory, ldcg at L2 only (never from L1), for kernels in which other CTAs of the
 // same launch overwrite the data between two reads. put: population stores to global memory
 // are evict-first: the next step reads them only after the whole lattice has gone by, and until
-// then they displace what neighbouring CTAs share in the L2 (256^3 FP32 with the spherical
-// sink: 1.18 against 1.08 ms per step).
+// then they can displace what neighbouring CTAs share in the L2. The difference is small since the
+// CTAs claim their work in order: evict-first / plain, us per step, shifted FP16 512 x 288 x 201 1752 /
+// 1765, FP32 256^3 with the spherical sink 969 / 967, 512^3 6889 / 6873.
 struct StF32 {
   using T = float2;
   static __device__ __forceinline__ float2 cv(T v, float) { return v; }
@@ -734,8 +738,8 @@ struct Tile {
 // Only the last right margin needs that; the others fetch theirs so that all tiles take
 // the same time: with the pieces at lattice edges alone, edge tiles ran 10% slower, fell
 // planes behind their neighbours, and the rows and 128-byte lines that neighbours share
-// were read from DRAM again (512^3 FP32, 64 x 4 tiles: 47 GB read per step against 23.7 GB,
-// 10.75 ms against 7.2 ms).
+// were read from DRAM again (224^3 FP32, 64 x 4 tiles: 2.62 GB read per step against 1.87, of 1.71
+// needed, 869 us against 664; with the spherical sink 955 against 714).
 //
 // Per plane: wait for the copies, read out plane p (Psi to the ring, own populations
 // to registers), barrier, start plane p + d's copies, collide plane p - d.

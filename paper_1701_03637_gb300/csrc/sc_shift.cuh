@@ -16,9 +16,11 @@
 // Why: in place, the force needs Psi of a neighbour before that neighbour is overwritten, so
 // the AA steps read every population twice, and on a 512^2 plane (40 MB per plane, three in
 // use) the second read misses the L2. Here it is read once, plus the halo planes of the chunks:
-// 512^3 FP32, 20 steps 234 (persistent) -> 184 ms, 9.2 ms per step against a floor of 6.0; what
-// is left beyond the two-lattice step's 7.3 ms is the chunks of 19 planes (two planes staged
-// for nothing per chunk) and a register spill in the march.
+// 512^3 FP32, 20 steps 234 (persistent) -> 180 ms, 9.0 ms per step against a floor of 6.0 and the
+// two-lattice step's 6.9 (a slower GPU of the kind took 215). Beyond that it reads more: 512 x 288 x 201
+// FP16, chunks of up to 15 planes, 3.3 to 3.4 GB per step for 2.25 needed, 1.28 times of it the
+// planes on each side of a chunk, the rest rows that neighbouring tiles no longer find in the
+// L2; it writes 2.27 GB. The march spills 94 bytes a thread (FP32 and scaled FP16; 90 FP16 and BF16).
 
 namespace {
 

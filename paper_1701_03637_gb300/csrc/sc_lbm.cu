@@ -244,6 +244,7 @@ struct AAPersist {
   float2* edge;                 // saved Psi columns: [k][nz][ny], k = b for band b's last column
                                 // (b < B - 1), k = B - 1 for band 0's first column
   int* err;                     // 0, or 1 + where a wait gave up
+  int* h_err;                   // the same for the host
   long long limit_ns;           // wait limit
   int withhold;                 // this CTA never reports its Psi planes (-1: none): makes its
                                 // neighbours' waits run out, to test the failure path
@@ -269,7 +270,7 @@ __device__ __forceinline__ bool poll_neighbour(const AAPersist& a, const unsigne
   const unsigned long long t0 = global_ns();
   while (ld_acquire_u64(p) < target) {
     if (*(volatile int*)a.err != 0 || (long long)(global_ns() - t0) > a.limit_ns) {
-      atomicCAS(a.err, 0, 1 + where);
+      if (atomicCAS(a.err, 0, 1 + where) == 0) *a.h_err = 1 + where;
       return false;
     }
   }
@@ -674,8 +675,7 @@ __device__ __align__(256) double g_noalloc_scratch[kNoAllocScratch];
 
 __global__ void k_diag_finish(const double* __restrict__ part, int nz, int nsplit, double nxy, int wall_z0,
                               int wall_z1, const double* __restrict__ evap_slots, long long nslots,
-                              double evap_offset, const int* __restrict__ persist_err, const int* __restrict__ err,
-                              double* __restrict__ out) {
+                              double evap_offset, const int* __restrict__ err, double* __restrict__ out) {
   if (blockIdx.x != 0 || threadIdx.x != 0) return;
   double mass_r = 0.0, mass_b = 0.0, pending = 0.0, count = 0.0, nonfinite = 0.0, sinkneg = 0.0;
   const int z0 = wall_z1 > wall_z0 ? wall_z1 : 0;
@@ -712,7 +712,7 @@ __global__ void k_diag_finish(const double* __restrict__ part, int nz, int nspli
   out[6] = count;
   const bool bad = nonfinite > 0.0 || !isfinite(mass_r) || !isfinite(mass_b);
   out[7] = bad ? (double)SC_ENONFINITE : (sinkneg > 0.0 ? (double)SC_ESINKNEG : (double)SC_OK);
-  if ((persist_err && *persist_err != 0) || *err != 0) out[7] = (double)SC_ETIMEOUT;
+  if (*err != 0) out[7] = (double)SC_ETIMEOUT;
 }
 
 // Initial / restored state: canonical populations of sites [s0, s1) from
@@ -1049,7 +1049,8 @@ struct sc_lbm {
   double evap_offset;  // evaporated mass restored by sc_lbm_set_counters
   double* h_diag;      // pinned
   double* h_evap;      // pinned
-  int* h_err;          // pinned, set by a step whose copies (3) or whose neighbours (4) did not come in time
+  int* h_err;          // pinned: 1, 2 a wait of the persistent step gave up, 3 a plane's copies, 4 a neighbour's
+                       // chunk did not come in time (shifted)
   CUtensorMap maps[2]; // of the two population buffers, with the tile's box (staged rows)
   int grid;  // CTAs of the persistent step (in place: of k_aa_collide)
   int grid_psi;  // CTAs of k_aa_psi
@@ -1393,6 +1394,7 @@ cudaError_t launch_persist_t(sc_lbm* h, int K, cudaStream_t st) {
   a.psi_done = h->flags();
   a.steps_done = h->flags() + kMaxCtas;
   a.err = h->err();
+  a.h_err = h->h_err;
   a.limit_ns = h->wait_limit_ns;
   a.withhold = h->withhold;
   LatDev L = h->L;
@@ -1421,19 +1423,12 @@ int launch_persist(sc_lbm* h, int K, cudaStream_t st) {
 // or of a step's plane copies gave up (the lattice's state is then undefined until it is loaded
 // again). Every call that hands the state to the host ends with it.
 int wait_status(sc_lbm* h) {
+  static const char* const what[] = {"a wait of the persistent in-place step gave up (between steps)",
+                                     "a wait of the persistent in-place step gave up (between planes)",
+                                     "a step's copies of a plane did not land in time",
+                                     "a wait of the shifted in-place step for its neighbours gave up"};
   const int e = *(volatile int*)h->h_err;
-  if (e != 0)
-    return fail(SC_ETIMEOUT, "%s; load a state to continue",
-                e == 4 ? "a wait of the shifted in-place step for its neighbours gave up"
-                       : "a step's copies of a plane did not land in time");
-  if (!h->persist) return SC_OK;
-  int v = 0;
-  CK(cudaMemcpyAsync(&v, h->err(), sizeof(int), cudaMemcpyDeviceToHost, h->stream));
-  CK(cudaStreamSynchronize(h->stream));
-  if (v != 0)
-    return fail(SC_ETIMEOUT, "a wait of the persistent in-place step gave up (%s); load a state to continue",
-                v == 1 ? "between steps" : "between planes");
-  return SC_OK;
+  return e == 0 ? SC_OK : fail(SC_ETIMEOUT, "%s; load a state to continue", what[std::min(std::max(e, 1), 4) - 1]);
 }
 
 int launch_shift_one(sc_lbm* h, cudaStream_t st);
@@ -2081,7 +2076,7 @@ int sc_lbm_diagnostics_noalloc(sc_lbm* h, double* out_dev) {
   if (rc) return rc;
   k_diag_finish<<<1, 1, 0, h->stream>>>(part, h->p.nz, h->lay.diag_nsplit, (double)h->p.nx * h->p.ny, h->L.wall_z0,
                                         h->L.wall_z1, h->evap(), h->lay.nslots, h->evap_offset,
-                                        h->persist ? h->err() : nullptr, h->h_err, out_dev);
+                                        h->h_err, out_dev);
   CK(cudaGetLastError());
   return SC_OK;
 }
